@@ -15,6 +15,7 @@
 #include "framefb_dense.h"
 #include "framefb_kernels.cuh"
 #include "framefb_mma.cuh"
+#include "framefb_row.h"
 #include "framefb_tc.cuh"
 #include "framefb_tc2.cuh"
 #include "framefb_tc2p.cuh"
@@ -722,7 +723,8 @@ bool parts_allowed() {
   return !(e && std::strcmp(e, "0") == 0);
 }
 
-// Matrices of a call split by path, each in call order: the fused kernels
+// Matrices of a call split by path, each in call order: the row-transform
+// kernel (framefb_row.cu), the fused kernels
 // (structured plans they take, fp32, or rows with padding), the plans' parts
 // on the fused tcgen05 kernels (bf16 structured plans the kernels do not
 // take whole, with parts, and tokens; FRAMEFB_PARTS=0 sends them to the
@@ -730,13 +732,18 @@ bool parts_allowed() {
 // (dense-layout plans, and the other bf16 structured plans the fused
 // tcgen05 kernels do not take, with unpadded rows).  FRAMEFB_KERNEL=tile
 // keeps every structured plan on the warp-MMA kernel.
-framefb_status split_paths(const framefb_mat* mats, int32_t nmats, framefb_dtype dt, std::vector<framefb_mat>& grp,
-                           std::vector<framefb_mat>& den, std::vector<framefb_mat>* prt = nullptr) {
+framefb_status split_paths(const framefb_mat* mats, int32_t nmats, int32_t ops, framefb_dtype dt,
+                           std::vector<framefb_mat>& grp, std::vector<framefb_mat>& den, std::vector<framefb_mat>& row,
+                           std::vector<framefb_mat>* prt = nullptr) {
   try {
     for (int32_t j = 0; j < nmats; ++j) {
       const framefb_mat& M = mats[j];
       const FfbPlanHeader* h = plan_header(M.plan);
       if (!h) return FRAMEFB_EINVAL;
+      if (ffb_host::row_takes(M, ops, dt)) {
+        row.push_back(M);
+        continue;
+      }
       const bool big = h->layout == FFB_LAYOUT_GROUPS && dt == FRAMEFB_BF16 && tc_allowed() && !fused_tc_ok(*h);
       if (big && prt && parts_allowed() && !M.plan->subs.empty() && M.N > 0) {
         prt->push_back(M);
@@ -767,9 +774,10 @@ framefb_status split_paths(const framefb_mat* mats, int32_t nmats, framefb_dtype
 // (backward dx) read-modify-write the same bytes and go to successive waves
 // (greedily), so that no launch holds both.
 framefb_status plan_waves(const framefb_mat* mats, int32_t nmats, int32_t ops, framefb_dtype dt,
-                          std::vector<std::vector<framefb_mat>>& waves, std::vector<framefb_mat>& den) {
+                          std::vector<std::vector<framefb_mat>>& waves, std::vector<framefb_mat>& den,
+                          std::vector<framefb_mat>& row) {
   std::vector<framefb_mat> grp, prt;
-  framefb_status s = split_paths(mats, nmats, dt, grp, den, &prt);
+  framefb_status s = split_paths(mats, nmats, ops, dt, grp, den, row, &prt);
   if (s != FRAMEFB_OK) return s;
   const bool F = ops & FRAMEFB_OP_FORWARD, D = ops & FRAMEFB_OP_BACKWARD_DX;
   const size_t esz = dt == FRAMEFB_BF16 ? 2 : 4;
@@ -818,13 +826,14 @@ extern "C" size_t framefb_workspace_size(const framefb_mat* mats, int32_t nmats,
   size_t need = 0;
   for (const framefb_dtype dt : {FRAMEFB_BF16, FRAMEFB_F32}) {
     std::vector<std::vector<framefb_mat>> waves;
-    std::vector<framefb_mat> den;
-    if (plan_waves(mats, nmats, ops, dt, waves, den) != FRAMEFB_OK) return 0;
-    size_t dneed = 0;
+    std::vector<framefb_mat> den, row;
+    if (plan_waves(mats, nmats, ops, dt, waves, den, row) != FRAMEFB_OK) return 0;
+    size_t dneed = 0, rneed = 0;
     if (!den.empty() &&
         ffb_host::dense_check(den.data(), static_cast<int32_t>(den.size()), ops, dt, &dneed) != FRAMEFB_OK)
       continue;
-    need = std::max(need, dneed);
+    if (ffb_host::row_check(row.data(), static_cast<int32_t>(row.size()), ops, dt, &rneed) != FRAMEFB_OK) continue;
+    need = std::max({need, dneed, rneed});
     for (const std::vector<framefb_mat>& w : waves)
       need = std::max(need, structured_workspace(w.data(), static_cast<int32_t>(w.size()), ops));
   }
@@ -838,8 +847,8 @@ extern "C" framefb_status framefb_run(const framefb_mat* mats, int32_t nmats, in
   if (nmats == 0) return FRAMEFB_OK;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   std::vector<std::vector<framefb_mat>> waves;
-  std::vector<framefb_mat> den;
-  framefb_status s = plan_waves(mats, nmats, ops, dtype, waves, den);
+  std::vector<framefb_mat> den, row;
+  framefb_status s = plan_waves(mats, nmats, ops, dtype, waves, den, row);
   if (s != FRAMEFB_OK) return s;
   // validate everything before queueing anything; the waves and the two
   // paths run one after the other on the stream and share the workspace
@@ -850,10 +859,12 @@ extern "C" framefb_status framefb_run(const framefb_mat* mats, int32_t nmats, in
     if (s != FRAMEFB_OK) return s;
     need = std::max(need, gneed);
   }
-  size_t dneed = 0;
+  size_t dneed = 0, rneed = 0;
   s = ffb_host::dense_check(den.data(), static_cast<int32_t>(den.size()), ops, dtype, &dneed);
   if (s != FRAMEFB_OK) return s;
-  need = std::max(need, dneed);
+  s = ffb_host::row_check(row.data(), static_cast<int32_t>(row.size()), ops, dtype, &rneed);
+  if (s != FRAMEFB_OK) return s;
+  need = std::max({need, dneed, rneed});
   if (need > 0) {
     if (!ws || ws_bytes < need) return FRAMEFB_EWORKSPACE;
     if (reinterpret_cast<uintptr_t>(ws) & 255u) return FRAMEFB_EINVAL;
@@ -862,6 +873,8 @@ extern "C" framefb_status framefb_run(const framefb_mat* mats, int32_t nmats, in
     s = structured_run(w.data(), static_cast<int32_t>(w.size()), ops, dtype, ws, st);
     if (s != FRAMEFB_OK) return s;
   }
+  s = ffb_host::row_run(row.data(), static_cast<int32_t>(row.size()), ops, dtype, ws, st);
+  if (s != FRAMEFB_OK) return s;
   return ffb_host::dense_run(den.data(), static_cast<int32_t>(den.size()), ops, dtype, ws, ws_bytes, st);
 }
 
@@ -872,12 +885,19 @@ extern "C" framefb_status framefb_kernel_names(const framefb_mat* mats, int32_t 
   if (nmats < 0 || (nmats > 0 && !mats) || !ops_ok(ops)) return FRAMEFB_EINVAL;
   if (dtype != FRAMEFB_F32 && dtype != FRAMEFB_BF16) return FRAMEFB_EINVAL;
   std::vector<std::vector<framefb_mat>> waves;
-  std::vector<framefb_mat> den;
-  framefb_status s = plan_waves(mats, nmats, ops, dtype, waves, den);
+  std::vector<framefb_mat> den, row;
+  framefb_status s = plan_waves(mats, nmats, ops, dtype, waves, den, row);
   if (s != FRAMEFB_OK) return s;
   std::vector<std::string> names;
   for (const std::vector<framefb_mat>& w : waves) {
     s = structured_names(w.data(), static_cast<int32_t>(w.size()), ops, dtype, names);
+    if (s != FRAMEFB_OK) return s;
+  }
+  if (!row.empty()) {
+    size_t need = 0;
+    s = ffb_host::row_check(row.data(), static_cast<int32_t>(row.size()), ops, dtype, &need);
+    if (s != FRAMEFB_OK) return s;
+    s = ffb_host::row_kernel_names(row.data(), static_cast<int32_t>(row.size()), ops, dtype, names);
     if (s != FRAMEFB_OK) return s;
   }
   if (!den.empty()) {
@@ -985,10 +1005,10 @@ extern "C" framefb_status framefb_forward_tenants(const framefb_mat* mats, int32
   // kernel (FRAMEFB_SEG_KERNEL=0 takes the per-segment path below)
   const char* env = std::getenv("FRAMEFB_SEG_KERNEL");
   if (dtype == FRAMEFB_BF16 && nmats > 0 && nseg > 0 && nseg <= ffb::kTcMaxSeg && !(env && std::strcmp(env, "0") == 0)) {
-    std::vector<framefb_mat> grp, den;
-    framefb_status s = split_paths(mats, nmats, dtype, grp, den);
+    std::vector<framefb_mat> grp, den, row;
+    framefb_status s = split_paths(mats, nmats, FRAMEFB_OP_FORWARD, dtype, grp, den, row);
     if (s != FRAMEFB_OK) return s;
-    if (den.empty()) {
+    if (den.empty() && row.empty()) {
       const SegTable st{nseg, seg_start, seg_tenant};
       size_t need = 0;
       s = structured_check(grp.data(), static_cast<int32_t>(grp.size()), FRAMEFB_OP_FORWARD, dtype, &need, &st);
@@ -1142,10 +1162,12 @@ extern "C" framefb_status framefb_run_static_ws(const framefb_mat* mats, int32_t
 
 extern "C" framefb_status framefb_wait_timeouts(uint32_t* count) {
   if (!count) return FRAMEFB_EINVAL;
-  uint32_t structured = 0, dense = 0;
+  uint32_t structured = 0, dense = 0, row = 0;
   if (cudaMemcpyFromSymbol(&structured, ffb::g_wait_timeouts, sizeof(uint32_t)) != cudaSuccess) return FRAMEFB_ECUDA;
   const framefb_status s = ffb_host::dense_wait_timeouts(&dense);
   if (s != FRAMEFB_OK) return s;
-  *count = structured + dense;
+  const framefb_status r = ffb_host::row_wait_timeouts(&row);
+  if (r != FRAMEFB_OK) return r;
+  *count = structured + dense + row;
   return FRAMEFB_OK;
 }

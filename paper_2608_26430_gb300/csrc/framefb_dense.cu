@@ -342,6 +342,11 @@ bool sy_maps(fd::GemmProblem& P, bool grouped, const float* R, int64_t ldr, int6
 
 }  // namespace
 
+bool dense_mat_ok(const framefb_mat& M, int32_t ops) {
+  const FfbPlanHeader* h = header_of(M.plan);
+  return h && check_mat(M, ops, *h);
+}
+
 framefb_status dense_check(const framefb_mat* mats, int32_t nmats, int32_t ops, framefb_dtype dt, size_t* ws_need) {
   *ws_need = 0;
   if (nmats == 0) return FRAMEFB_OK;

@@ -23,6 +23,10 @@ EncodeTiledFn encode_tiled();
 // another and share it).
 framefb_status dense_check(const framefb_mat* mats, int32_t nmats, int32_t ops, framefb_dtype dt, size_t* ws_need);
 
+// The argument checks of dense_check on one matrix (bf16; rows, pointers,
+// frames and plan of its path).
+bool dense_mat_ok(const framefb_mat& M, int32_t ops);
+
 // Queue the dense path of every matrix on `st` (after dense_check).
 framefb_status dense_run(const framefb_mat* mats, int32_t nmats, int32_t ops, framefb_dtype dt, void* ws,
                          size_t ws_bytes, cudaStream_t st);
