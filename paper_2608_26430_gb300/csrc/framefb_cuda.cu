@@ -13,6 +13,7 @@
 
 #include "framefb.h"
 #include "framefb_dense.h"
+#include "framefb_grp.h"
 #include "framefb_kernels.cuh"
 #include "framefb_mma.cuh"
 #include "framefb_row.h"
@@ -734,6 +735,7 @@ bool parts_allowed() {
 // keeps every structured plan on the warp-MMA kernel.
 framefb_status split_paths(const framefb_mat* mats, int32_t nmats, int32_t ops, framefb_dtype dt,
                            std::vector<framefb_mat>& grp, std::vector<framefb_mat>& den, std::vector<framefb_mat>& row,
+                           std::vector<framefb_mat>& fft,
                            std::vector<framefb_mat>* prt = nullptr) {
   try {
     for (int32_t j = 0; j < nmats; ++j) {
@@ -742,6 +744,10 @@ framefb_status split_paths(const framefb_mat* mats, int32_t nmats, int32_t ops, 
       if (!h) return FRAMEFB_EINVAL;
       if (ffb_host::row_takes(M, ops, dt)) {
         row.push_back(M);
+        continue;
+      }
+      if (tc_allowed() && ffb_host::grp_takes(M, ops, dt)) {
+        fft.push_back(M);
         continue;
       }
       const bool big = h->layout == FFB_LAYOUT_GROUPS && dt == FRAMEFB_BF16 && tc_allowed() && !fused_tc_ok(*h);
@@ -775,9 +781,9 @@ framefb_status split_paths(const framefb_mat* mats, int32_t nmats, int32_t ops, 
 // (greedily), so that no launch holds both.
 framefb_status plan_waves(const framefb_mat* mats, int32_t nmats, int32_t ops, framefb_dtype dt,
                           std::vector<std::vector<framefb_mat>>& waves, std::vector<framefb_mat>& den,
-                          std::vector<framefb_mat>& row) {
+                          std::vector<framefb_mat>& row, std::vector<framefb_mat>& fft) {
   std::vector<framefb_mat> grp, prt;
-  framefb_status s = split_paths(mats, nmats, ops, dt, grp, den, row, &prt);
+  framefb_status s = split_paths(mats, nmats, ops, dt, grp, den, row, fft, &prt);
   if (s != FRAMEFB_OK) return s;
   const bool F = ops & FRAMEFB_OP_FORWARD, D = ops & FRAMEFB_OP_BACKWARD_DX;
   const size_t esz = dt == FRAMEFB_BF16 ? 2 : 4;
@@ -826,14 +832,16 @@ extern "C" size_t framefb_workspace_size(const framefb_mat* mats, int32_t nmats,
   size_t need = 0;
   for (const framefb_dtype dt : {FRAMEFB_BF16, FRAMEFB_F32}) {
     std::vector<std::vector<framefb_mat>> waves;
-    std::vector<framefb_mat> den, row;
-    if (plan_waves(mats, nmats, ops, dt, waves, den, row) != FRAMEFB_OK) return 0;
+    std::vector<framefb_mat> den, row, fft;
+    if (plan_waves(mats, nmats, ops, dt, waves, den, row, fft) != FRAMEFB_OK) return 0;
     size_t dneed = 0, rneed = 0;
     if (!den.empty() &&
         ffb_host::dense_check(den.data(), static_cast<int32_t>(den.size()), ops, dt, &dneed) != FRAMEFB_OK)
       continue;
     if (ffb_host::row_check(row.data(), static_cast<int32_t>(row.size()), ops, dt, &rneed) != FRAMEFB_OK) continue;
-    need = std::max({need, dneed, rneed});
+    size_t fneed = 0;
+    if (ffb_host::grp_check(fft.data(), static_cast<int32_t>(fft.size()), ops, dt, &fneed) != FRAMEFB_OK) continue;
+    need = std::max({need, dneed, rneed, fneed});
     for (const std::vector<framefb_mat>& w : waves)
       need = std::max(need, structured_workspace(w.data(), static_cast<int32_t>(w.size()), ops));
   }
@@ -847,8 +855,8 @@ extern "C" framefb_status framefb_run(const framefb_mat* mats, int32_t nmats, in
   if (nmats == 0) return FRAMEFB_OK;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   std::vector<std::vector<framefb_mat>> waves;
-  std::vector<framefb_mat> den, row;
-  framefb_status s = plan_waves(mats, nmats, ops, dtype, waves, den, row);
+  std::vector<framefb_mat> den, row, fft;
+  framefb_status s = plan_waves(mats, nmats, ops, dtype, waves, den, row, fft);
   if (s != FRAMEFB_OK) return s;
   // validate everything before queueing anything; the waves and the two
   // paths run one after the other on the stream and share the workspace
@@ -864,7 +872,10 @@ extern "C" framefb_status framefb_run(const framefb_mat* mats, int32_t nmats, in
   if (s != FRAMEFB_OK) return s;
   s = ffb_host::row_check(row.data(), static_cast<int32_t>(row.size()), ops, dtype, &rneed);
   if (s != FRAMEFB_OK) return s;
-  need = std::max({need, dneed, rneed});
+  size_t fneed = 0;
+  s = ffb_host::grp_check(fft.data(), static_cast<int32_t>(fft.size()), ops, dtype, &fneed);
+  if (s != FRAMEFB_OK) return s;
+  need = std::max({need, dneed, rneed, fneed});
   if (need > 0) {
     if (!ws || ws_bytes < need) return FRAMEFB_EWORKSPACE;
     if (reinterpret_cast<uintptr_t>(ws) & 255u) return FRAMEFB_EINVAL;
@@ -873,6 +884,8 @@ extern "C" framefb_status framefb_run(const framefb_mat* mats, int32_t nmats, in
     s = structured_run(w.data(), static_cast<int32_t>(w.size()), ops, dtype, ws, st);
     if (s != FRAMEFB_OK) return s;
   }
+  s = ffb_host::grp_run(fft.data(), static_cast<int32_t>(fft.size()), ops, dtype, ws, st);
+  if (s != FRAMEFB_OK) return s;
   s = ffb_host::row_run(row.data(), static_cast<int32_t>(row.size()), ops, dtype, ws, st);
   if (s != FRAMEFB_OK) return s;
   return ffb_host::dense_run(den.data(), static_cast<int32_t>(den.size()), ops, dtype, ws, ws_bytes, st);
@@ -885,13 +898,20 @@ extern "C" framefb_status framefb_kernel_names(const framefb_mat* mats, int32_t 
   if (nmats < 0 || (nmats > 0 && !mats) || !ops_ok(ops)) return FRAMEFB_EINVAL;
   if (dtype != FRAMEFB_F32 && dtype != FRAMEFB_BF16) return FRAMEFB_EINVAL;
   std::vector<std::vector<framefb_mat>> waves;
-  std::vector<framefb_mat> den, row;
-  framefb_status s = plan_waves(mats, nmats, ops, dtype, waves, den, row);
+  std::vector<framefb_mat> den, row, fft;
+  framefb_status s = plan_waves(mats, nmats, ops, dtype, waves, den, row, fft);
   if (s != FRAMEFB_OK) return s;
   std::vector<std::string> names;
   for (const std::vector<framefb_mat>& w : waves) {
     s = structured_names(w.data(), static_cast<int32_t>(w.size()), ops, dtype, names);
     if (s != FRAMEFB_OK) return s;
+  }
+  if (!fft.empty()) {
+    size_t need = 0;
+    s = ffb_host::grp_check(fft.data(), static_cast<int32_t>(fft.size()), ops, dtype, &need);
+    if (s != FRAMEFB_OK) return s;
+    const std::string k = "fft_tile_kernel<" + std::to_string(ops) + ">";
+    if (std::find(names.begin(), names.end(), k) == names.end()) names.push_back(k);
   }
   if (!row.empty()) {
     size_t need = 0;
@@ -1005,10 +1025,10 @@ extern "C" framefb_status framefb_forward_tenants(const framefb_mat* mats, int32
   // kernel (FRAMEFB_SEG_KERNEL=0 takes the per-segment path below)
   const char* env = std::getenv("FRAMEFB_SEG_KERNEL");
   if (dtype == FRAMEFB_BF16 && nmats > 0 && nseg > 0 && nseg <= ffb::kTcMaxSeg && !(env && std::strcmp(env, "0") == 0)) {
-    std::vector<framefb_mat> grp, den, row;
-    framefb_status s = split_paths(mats, nmats, FRAMEFB_OP_FORWARD, dtype, grp, den, row);
+    std::vector<framefb_mat> grp, den, row, fft;
+    framefb_status s = split_paths(mats, nmats, FRAMEFB_OP_FORWARD, dtype, grp, den, row, fft);
     if (s != FRAMEFB_OK) return s;
-    if (den.empty() && row.empty()) {
+    if (den.empty() && row.empty() && fft.empty()) {
       const SegTable st{nseg, seg_start, seg_tenant};
       size_t need = 0;
       s = structured_check(grp.data(), static_cast<int32_t>(grp.size()), FRAMEFB_OP_FORWARD, dtype, &need, &st);

@@ -1,0 +1,398 @@
+// Launchers of the group-transform path of libframefb (framefb_grp.cuh): which
+// structured matrices it takes, validation, the shared-memory map, launches.
+#include <cuda_bf16.h>
+#include <cuda_runtime.h>
+
+#include <algorithm>
+#include <cmath>
+#include <cstring>
+#include <memory>
+#include <new>
+#include <string>
+#include <vector>
+
+#include "framefb.h"
+#include "framefb_grp.cuh"
+#include "framefb_grp.h"
+#include "plan_internal.h"
+#include "plan_layout.h"
+
+namespace ffb_host {
+
+namespace {
+
+namespace fg = ffb::grp;
+namespace fp = ffb::pair;
+
+static_assert(sizeof(fg::Launch) <= 32764 && sizeof(fp::Reduce) <= 32764, "launch parameters exceed the parameter space");
+static_assert(fg::kMaxMats <= fp::kReduceMats, "one reduction per launch");
+
+inline size_t rup(size_t x, size_t a) { return (x + a - 1) / a * a; }
+inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
+
+const FfbPlanHeader* header_of(const framefb_plan* p) {
+  if (!p || p->image.size() < sizeof(FfbPlanHeader)) return nullptr;
+  const FfbPlanHeader* h = reinterpret_cast<const FfbPlanHeader*>(p->image.data());
+  if (h->magic != FFB_PLAN_MAGIC || h->version != FFB_PLAN_VERSION || h->P != fp::kColumns) return nullptr;
+  if (static_cast<size_t>(h->total_bytes) > p->image.size() || h->layout != FFB_LAYOUT_GROUPS) return nullptr;
+  return h;
+}
+
+// A kernel variant: threads per CTA, plan entries per thread and path, big
+// plans (compacted buffers).
+struct Variant {
+  int nt, ke;
+  bool big;
+  bool operator==(const Variant& o) const { return nt == o.nt && ke == o.ke && big == o.big; }
+};
+
+constexpr size_t kSmemSm = 228 * 1024;          // shared memory of an SM
+constexpr size_t kSmemCta = 227 * 1024 - 256;   // of a CTA, less the static part
+constexpr int kMaxPairs = 8;
+// relative cost of a group's transform and of a support entry (per pair)
+constexpr int kGroupCost = 16, kEntryCost = 1;
+
+size_t budget(const Variant& v) { return v.nt == 512 ? kSmemCta : kSmemSm / 2 - 1024 - 256; }
+
+// Columns of a side in the support (set bits of the plan's group masks).
+int32_t named(const FfbPlanHeader* h, int sd) {
+  const uint8_t* base = reinterpret_cast<const uint8_t*>(h);
+  const uint32_t* m = reinterpret_cast<const uint32_t*>(base + (sd ? h->off_zmask : h->off_gmask));
+  int32_t n = 0;
+  for (int32_t g = 0; g < (sd ? h->Gm : h->Gn); ++g) n += __builtin_popcount(m[g]);
+  return n;
+}
+
+// Buffers of a token pair of a matrix on a variant; false when slots exceed
+// the variant's fields.
+bool shape_of(const FfbPlanHeader* h, const Variant& v, fg::Shape& sh) {
+  std::memset(&sh, 0, sizeof(sh));
+  int32_t off = 0;
+  for (int sd = 0; sd < 2; ++sd) {
+    const int32_t d = sd ? h->m : h->n, ovf = sd ? h->ovfZ : h->ovfG;
+    const int32_t slots = v.big ? named(h, sd) : d;
+    if (v.big ? slots + ovf > (sd ? fg::kBigU : fg::kBigV) : slots + ovf > fp::kMaxSlots) return false;
+    sh.G[sd] = d / FFB_GROUP;
+    sh.A[sd] = off;
+    off += static_cast<int32_t>(rup(std::max(slots, 1), 2));
+    sh.B[sd] = off;
+    off += static_cast<int32_t>(rup(std::max(slots + ovf, 1), 2));
+  }
+  sh.pair = off;
+  return true;
+}
+
+// Shared memory of a launch: the largest of its shapes.
+struct Regions {
+  size_t pairs = 0, masks = 0;
+  void take(const fg::Shape& sh, int pp, const Variant& v) {
+    pairs = std::max(pairs, rup(static_cast<size_t>(pp) * sh.pair * 8, 16));
+    masks = std::max(masks, rup(4 * static_cast<size_t>((v.big ? 2 : 1) * (sh.G[0] + sh.G[1]) + 2), 16));
+  }
+  size_t plan(const Variant& v) const { return v.big ? fg::big_bytes(v.nt) : fg::cols_bytes(v.nt, v.ke); }
+  size_t bytes(const Variant& v) const { return pairs + masks + plan(v); }
+};
+
+// The kernel variant of a plan (nt = 0: none fits): two CTAs of 256 threads
+// per SM where a unit fits half an SM and a column has at most 8 entries, else
+// one CTA of 512 threads, with compacted buffers for columns of up to 32.
+Variant variant(const FfbPlanHeader* h) {
+  const int e = std::max(h->EZ, h->EG);
+  for (const Variant& v : {Variant{256, 4, false}, Variant{256, 8, false}, Variant{512, 8, false}, Variant{512, fg::kBigE, true}}) {
+    if (e > v.ke * (v.nt / fp::kColumns)) continue;
+    fg::Shape sh;
+    if (!shape_of(h, v, sh)) continue;
+    Regions r;
+    r.take(sh, 1, v);
+    if (r.bytes(v) <= budget(v)) return v;
+  }
+  return Variant{0, 0, false};
+}
+
+void* kernel_ptr(const Variant& v, framefb_dtype dt) {
+#define FFB_GRP(N, E, B)                                                                             \
+  if (v == Variant{N, E, B})                                                                         \
+    return dt == FRAMEFB_BF16 ? reinterpret_cast<void*>(fg::group_kernel<__nv_bfloat16, N, E, B>)    \
+                              : reinterpret_cast<void*>(fg::group_kernel<float, N, E, B>);
+  FFB_GRP(256, 4, false)
+  FFB_GRP(256, 8, false)
+  FFB_GRP(512, 8, false)
+  FFB_GRP(512, fg::kBigE, true)
+#undef FFB_GRP
+  return nullptr;
+}
+
+struct Prepared {
+  fg::Launch* args;
+  fp::Reduce* red;
+  int grid, nnz_max;
+  Variant v;
+  size_t smem, ws_bytes;
+};
+
+// One launch: as many matrices as the parameters hold, of one variant.
+struct Chunk {
+  std::vector<const framefb_mat*> mats;
+  Variant v;
+};
+
+std::vector<Chunk> chunks_of(const framefb_mat* mats, int32_t nmats) {
+  std::vector<Variant> kinds;
+  std::vector<Variant> of(nmats);
+  for (int32_t j = 0; j < nmats; ++j) {
+    // (matrices of one plan come in runs)
+    of[j] = j > 0 && mats[j].plan == mats[j - 1].plan ? of[j - 1] : variant(header_of(mats[j].plan));
+    if (of[j].nt && std::find(kinds.begin(), kinds.end(), of[j]) == kinds.end()) kinds.push_back(of[j]);
+  }
+  std::vector<Chunk> out;
+  for (const Variant& v : kinds) {
+    std::vector<const FfbPlanHeader*> shapes;
+    Regions all;  // of one pair of each shape of the chunk
+    bool open = false;
+    for (int32_t j = 0; j < nmats; ++j) {
+      if (!(of[j] == v)) continue;
+      const FfbPlanHeader* h = header_of(mats[j].plan);
+      bool known = std::find(shapes.begin(), shapes.end(), h) != shapes.end();
+      fg::Shape sh;
+      Regions with = all;
+      if (!known) {
+        shape_of(h, v, sh);
+        with.take(sh, 1, v);
+      }
+      if (!open || static_cast<int>(out.back().mats.size()) == fg::kMaxMats ||
+          (!known && (static_cast<int>(shapes.size()) == fg::kMaxShapes || with.bytes(v) > budget(v)))) {
+        out.push_back(Chunk{{}, v});
+        shapes.clear();
+        all = Regions();
+        open = true;
+        if (known) shape_of(h, v, sh);
+        known = false;
+      }
+      if (!known) {
+        shapes.push_back(h);
+        all.take(sh, 1, v);
+      }
+      out.back().mats.push_back(&mats[j]);
+    }
+  }
+  return out;
+}
+
+framefb_status prepare(const Chunk& ch, int32_t ops, framefb_dtype dt, Prepared& P) {
+  std::memset(P.args, 0, sizeof(fg::Launch));
+  std::memset(P.red, 0, sizeof(fp::Reduce));
+  fg::Launch& A = *P.args;
+  P.v = ch.v;
+  void* fn = kernel_ptr(ch.v, dt);
+  if (!fn) return FRAMEFB_EINVAL;
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return FRAMEFB_ECUDA;
+  const int per = ch.v.nt == 512 ? 1 : 2;
+  const int nm = static_cast<int>(ch.mats.size());
+  // pairs per unit: what fits, but no more than gives every CTA a unit
+  int64_t pairs = 0;
+  for (const framefb_mat* M : ch.mats) pairs += (M->N + 1) / 2;
+  const int64_t spread = std::max<int64_t>(1, pairs / (static_cast<int64_t>(sms) * per));
+  std::vector<const FfbPlanHeader*> hd;
+  int nsh = 0;
+  Regions reg;
+  for (int j = 0; j < nm; ++j) {
+    const FfbPlanHeader* h = header_of(ch.mats[j]->plan);
+    const int s = static_cast<int>(std::find(hd.begin(), hd.end(), h) - hd.begin());
+    if (s == nsh) {
+      if (nsh == fg::kMaxShapes) return FRAMEFB_EINVAL;
+      hd.push_back(h);
+      fg::Shape& sh = A.sh[nsh++];
+      if (!shape_of(h, ch.v, sh)) return FRAMEFB_EINVAL;
+      reg.take(sh, 1, ch.v);
+    }
+    A.m[j].shape = s;
+  }
+  if (reg.bytes(ch.v) > budget(ch.v)) return FRAMEFB_EUNSUPPORTED;
+  const size_t room = budget(ch.v) - reg.masks - reg.plan(ch.v);
+  for (int i = 0; i < nsh; ++i) {
+    fg::Shape& sh = A.sh[i];
+    const int64_t fit = static_cast<int64_t>(room / (static_cast<size_t>(sh.pair) * 8));
+    sh.PP = static_cast<int32_t>(std::max<int64_t>(1, std::min<int64_t>({kMaxPairs, spread, fit})));
+    reg.take(sh, sh.PP, ch.v);
+  }
+  P.smem = reg.bytes(ch.v);
+  A.oPlan = static_cast<int32_t>(reg.pairs);
+  A.oMask = static_cast<int32_t>(reg.pairs + reg.plan(ch.v));
+  int64_t units = 0;
+  int32_t nnz_max = 0;
+  for (int j = 0; j < nm; ++j) {
+    const framefb_mat& M = *ch.mats[j];
+    const FfbPlanHeader& h = *header_of(M.plan);
+    fg::Mat& K = A.m[j];
+    const fg::Shape& sh = A.sh[K.shape];
+    K.in[0] = M.X;
+    K.in[1] = M.dY;
+    K.out[0] = M.dX;
+    K.out[1] = M.Y;
+    K.ld[0] = M.ldx;
+    K.ld[1] = M.ldy;
+    K.plan = static_cast<const uint8_t*>(M.plan_dev);
+    K.c_val = M.c_val;
+    K.N = M.N;
+    K.ubeg = static_cast<int32_t>(units);
+    K.ntiles = (M.N + 2 * sh.PP - 1) / (2 * sh.PP);
+    K.seff = static_cast<float>(static_cast<double>(M.scale) / 16.0);
+    // a unit's cost: groups to transform and entries to gather, per pair
+    K.cost = sh.PP * (2 * (h.Gn + h.Gm) * kGroupCost + h.nnz * kEntryCost) / 64 + 1;
+    K.cbeg = A.total_cost;
+    A.total_cost += static_cast<int64_t>(K.cost) * K.ntiles;
+    units += K.ntiles;
+    if (units > INT32_MAX / 2) return FRAMEFB_EUNSUPPORTED;
+    nnz_max = std::max(nnz_max, h.nnz);
+  }
+  A.nmats = nm;
+  A.mode = ops;
+  A.total_units = static_cast<int32_t>(units);
+  A.stride = (nnz_max + 63) & ~63;
+  P.nnz_max = nnz_max;
+  int per_sm = 0;
+  if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(P.smem)) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, ch.v.nt, P.smem) != cudaSuccess)
+    return FRAMEFB_ECUDA;
+  if (per_sm < 1) return FRAMEFB_EUNSUPPORTED;
+  // every CTA gets a unit: its share of the cost is at least the largest unit's
+  // (the dC reduction sums the slots of a matrix's first to last CTA)
+  int32_t max_cost = 1;
+  for (int j = 0; j < nm; ++j) max_cost = std::max(max_cost, A.m[j].ntiles > 0 ? A.m[j].cost : 1);
+  P.grid = static_cast<int>(std::min({static_cast<int64_t>(sms) * per_sm, units, A.total_cost / max_cost}));
+  P.ws_bytes = 0;
+  if (ops & FRAMEFB_OP_GRAD_COEFF) {
+    P.ws_bytes = static_cast<size_t>(P.grid + nm) * A.stride * sizeof(float) + 256;
+    P.red->stride = A.stride;
+    // CTA of unit u: the last one whose first unit is not past it
+    int32_t c = 0;
+    auto cta_of = [&](int32_t u) {
+      while (c + 1 < P.grid && fg::first_unit(A, c + 1, P.grid) <= u) ++c;
+      return c;
+    };
+    for (int j = 0; j < nm; ++j) {
+      fp::ReduceMat& R = P.red->m[j];
+      R.dC = ch.mats[j]->dC;
+      R.nnz = header_of(ch.mats[j]->plan)->nnz;
+      R.seff = A.m[j].seff;
+      R.c0 = cta_of(A.m[j].ubeg);
+      R.c1 = cta_of(A.m[j].ubeg + A.m[j].ntiles - 1);
+    }
+  }
+  return FRAMEFB_OK;
+}
+
+// Launch parameters live on the heap: too large for the stack of some callers.
+struct Buffers {
+  std::unique_ptr<fg::Launch> a{new fg::Launch};
+  std::unique_ptr<fp::Reduce> r{new fp::Reduce};
+  Prepared prep() {
+    Prepared p{};
+    p.args = a.get();
+    p.red = r.get();
+    return p;
+  }
+};
+
+
+bool frame_ok(const framefb_dev_frame* f, int32_t d) {
+  return f && f->dft_groups && f->k == 16 && f->d == d && f->ncols == d && f->rho * 16 == d && f->val && f->colptr && f->rowidx;
+}
+
+framefb_status check_mat(const framefb_mat& M, int32_t ops, framefb_dtype dt) {
+  const bool F = ops & FRAMEFB_OP_FORWARD, D = ops & FRAMEFB_OP_BACKWARD_DX, C = ops & FRAMEFB_OP_GRAD_COEFF;
+  const FfbPlanHeader* h = header_of(M.plan);
+  if (!h || M.N < 0 || M.n <= 0 || M.m <= 0 || h->n != M.n || h->m != M.m) return FRAMEFB_EINVAL;
+  if (!frame_ok(M.fin, M.n) || !frame_ok(M.fout, M.m)) return FRAMEFB_EINVAL;
+  if (!M.plan_dev || !aligned16(M.plan_dev) || !std::isfinite(M.scale)) return FRAMEFB_EINVAL;
+  if ((F || D) && h->nnz > 0 && !M.c_val) return FRAMEFB_EINVAL;
+  if (C && h->nnz > 0 && !M.dC) return FRAMEFB_EINVAL;
+  if (M.N == 0) return FRAMEFB_OK;
+  const int64_t esz = dt == FRAMEFB_BF16 ? 2 : 4;
+  const bool needX = F || C, needdY = D || C;
+  if ((needX || D) && (M.ldx < M.n || (M.ldx * esz) % 16)) return FRAMEFB_EINVAL;
+  if ((needdY || F) && (M.ldy < M.m || (M.ldy * esz) % 16)) return FRAMEFB_EINVAL;
+  if (needX && (!M.X || !aligned16(M.X))) return FRAMEFB_EINVAL;
+  if (needdY && (!M.dY || !aligned16(M.dY))) return FRAMEFB_EINVAL;
+  if (F && (!M.Y || !aligned16(M.Y))) return FRAMEFB_EINVAL;
+  if (D && (!M.dX || !aligned16(M.dX))) return FRAMEFB_EINVAL;
+  return FRAMEFB_OK;
+}
+
+}  // namespace
+
+// The path takes
+//   * fp32: every structured plan that fits a variant (the one-phase FFT kernel
+//     keeps the others).  Fused pass, that kernel -> this one: 8 matrices of
+//     768^2, 2048 tokens 203 -> 107 us; 2 of 3072^2, 1000 tokens 85 -> 63 us; 8 of
+//     256^2, 4096 tokens 277 -> 90 us; 8 tokens of one of 256^2 the same 21 us.
+//   * bf16: plans beyond the tcgen05 kernels with a side of more than 128
+//     groups (the LLaMA-3 MLP shapes), whole: the tcgen05 kernel would run them
+//     in parts or not at all.  8192 Zipf entries, fused, 64 / 1024 / 4096 tokens:
+//     4096 -> 14336 (five parts) 115 / 194 / 408 -> 49 / 102 / 249 us;
+//     14336 -> 4096 (contraction path) 61 / 220 / 664 -> 61 / 112 / 268 us, so
+//     that side from 128 tokens.  Narrower big plans stay in parts (4096^2, 8192
+//     tokens 289 us against 340 here).
+constexpr int32_t kMinTokensWideIn = 128;
+
+bool grp_takes(const framefb_mat& M, int32_t ops, framefb_dtype dt) {
+  (void)ops;
+  const FfbPlanHeader* h = header_of(M.plan);
+  if (!h || M.N < 1) return false;
+  const Variant v = variant(h);
+  if (v.nt == 0) return false;
+  if (dt == FRAMEFB_F32) return true;
+  return v.big && (h->Gm > 128 || (h->Gn > 128 && M.N >= kMinTokensWideIn));
+}
+
+framefb_status grp_check(const framefb_mat* mats, int32_t nmats, int32_t ops, framefb_dtype dt, size_t* ws_need) {
+  *ws_need = 0;
+  if (nmats == 0) return FRAMEFB_OK;
+  for (int32_t j = 0; j < nmats; ++j) {
+    const framefb_status s = check_mat(mats[j], ops, dt);
+    if (s != FRAMEFB_OK) return s;
+  }
+  try {
+    Buffers b;
+    for (const Chunk& c : chunks_of(mats, nmats)) {
+      Prepared P = b.prep();
+      const framefb_status s = prepare(c, ops, dt, P);
+      if (s != FRAMEFB_OK) return s;
+      *ws_need = std::max(*ws_need, P.ws_bytes);
+    }
+  } catch (const std::bad_alloc&) {
+    return FRAMEFB_ENOMEM;
+  }
+  return FRAMEFB_OK;
+}
+
+framefb_status grp_run(const framefb_mat* mats, int32_t nmats, int32_t ops, framefb_dtype dt, void* ws, cudaStream_t st) {
+  if (nmats == 0) return FRAMEFB_OK;
+  try {
+    Buffers b;
+    for (const Chunk& c : chunks_of(mats, nmats)) {
+      Prepared P = b.prep();
+      const framefb_status s = prepare(c, ops, dt, P);
+      if (s != FRAMEFB_OK) return s;
+      P.args->partial = static_cast<float*>(ws);
+      P.red->partial = static_cast<const float*>(ws);
+      void* kargs[] = {P.args};
+      if (cudaLaunchKernel(kernel_ptr(P.v, dt), dim3(P.grid), dim3(P.v.nt), kargs, P.smem, st) != cudaSuccess)
+        return FRAMEFB_ECUDA;
+      if ((ops & FRAMEFB_OP_GRAD_COEFF) && P.nnz_max > 0) {
+        void* rargs[] = {P.red};
+        if (cudaLaunchKernel(reinterpret_cast<void*>(fp::pair_reduce_kernel),
+                             dim3((P.nnz_max + 31) / 32, static_cast<unsigned>(c.mats.size())), dim3(32 * fp::kLanes), rargs,
+                             0, st) != cudaSuccess)
+          return FRAMEFB_ECUDA;
+      }
+    }
+  } catch (const std::bad_alloc&) {
+    return FRAMEFB_ENOMEM;
+  }
+  return FRAMEFB_OK;
+}
+
+}  // namespace ffb_host

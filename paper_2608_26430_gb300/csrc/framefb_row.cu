@@ -23,16 +23,18 @@ namespace ffb_host {
 
 namespace {
 
+namespace fp = ffb::pair;
 namespace fr = ffb::row;
+static_assert(fr::kMaxMats <= fp::kReduceMats, "one reduction per launch");
 
-static_assert(sizeof(fr::Launch) <= 32764 && sizeof(fr::Reduce) <= 32764, "launch parameters exceed the parameter space");
+static_assert(sizeof(fr::Launch) <= 32764 && sizeof(fp::Reduce) <= 32764, "launch parameters exceed the parameter space");
 
 inline size_t rup(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 const FfbPlanHeader* header_of(const framefb_plan* p) {
   if (!p || p->image.size() < sizeof(FfbPlanHeader)) return nullptr;
   const FfbPlanHeader* h = reinterpret_cast<const FfbPlanHeader*>(p->image.data());
-  if (h->magic != FFB_PLAN_MAGIC || h->version != FFB_PLAN_VERSION || h->P != fr::kColumns) return nullptr;
+  if (h->magic != FFB_PLAN_MAGIC || h->version != FFB_PLAN_VERSION || h->P != fp::kColumns) return nullptr;
   if (static_cast<size_t>(h->total_bytes) > p->image.size()) return nullptr;
   return h;
 }
@@ -57,6 +59,7 @@ bool shape_of(const framefb_mat& M, fr::Shape& sh) {
     off += scratch;
     sh.B[sd] = off;
     off += (std::max(K[sd] + ovf[sd], scratch) + 1) / 2 * 2;
+    if (K[sd] + ovf[sd] > fp::kMaxSlots) return false;
   }
   sh.pair = off;
   return true;
@@ -91,7 +94,7 @@ struct Regions {
     pairs = std::max(pairs, static_cast<size_t>(pp) * sh.pair * 8);
     tw = std::max(tw, rup(static_cast<size_t>(twiddles(sh)) * 8, 128));
   }
-  size_t bytes(const Variant& v) const { return stage[0] + stage[1] + pairs + tw + fr::plan_bytes(v.nt, v.ke) + 16; }
+  size_t bytes(const Variant& v) const { return stage[0] + stage[1] + pairs + tw + fp::plan_bytes(v.nt, v.ke) + 16; }
 };
 
 // Bytes a unit of `pp` pairs of a shape needs in all.
@@ -109,7 +112,7 @@ Variant variant(const framefb_mat& M, const fr::Shape& sh) {
   const int e = std::max(h.EZ, h.EG);
   const int k = sh.k[0] != sh.k[1] ? 0 : sh.k[0];
   for (const Variant& v : {Variant{256, 4, 0}, Variant{256, 8, 0}, Variant{512, 8, 0}}) {
-    if (e > v.ke * (v.nt / fr::kColumns) || unit_bytes(sh, 1, v) > budget(v.nt)) continue;
+    if (e > v.ke * (v.nt / fp::kColumns) || unit_bytes(sh, 1, v) > budget(v.nt)) continue;
     const bool own = v.nt == 512 ? k == 1024 || k == 2048 : k == 384 || k == 512;  // sizes with a kernel of their own
     return Variant{v.nt, v.ke, own ? k : 0};
   }
@@ -134,7 +137,7 @@ void* kernel_ptr(const Variant& v) {
 
 struct Prepared {
   fr::Launch* args;
-  fr::Reduce* red;
+  fp::Reduce* red;
   int grid, nnz_max;
   Variant v;
   size_t smem, ws_bytes;
@@ -185,7 +188,7 @@ std::vector<Chunk> chunks_of(const framefb_mat* mats, int32_t nmats) {
 
 framefb_status prepare(const Chunk& ch, int32_t ops, Prepared& P) {
   std::memset(P.args, 0, sizeof(fr::Launch));
-  std::memset(P.red, 0, sizeof(fr::Reduce));
+  std::memset(P.red, 0, sizeof(fp::Reduce));
   fr::Launch& A = *P.args;
   P.v = ch.v;
   void* fn = kernel_ptr(ch.v);
@@ -236,7 +239,7 @@ framefb_status prepare(const Chunk& ch, int32_t ops, Prepared& P) {
   A.oPairs = static_cast<int32_t>(reg.stage[0] + reg.stage[1]);
   A.oTw = static_cast<int32_t>(A.oPairs + reg.pairs);
   A.oPlan = static_cast<int32_t>(A.oTw + reg.tw);
-  A.oBar = A.oPlan + fr::plan_bytes(ch.v.nt, ch.v.ke);
+  A.oBar = A.oPlan + fp::plan_bytes(ch.v.nt, ch.v.ke);
   int64_t units = 0;
   int32_t nnz_max = 0;
   for (int j = 0; j < nm; ++j) {
@@ -277,7 +280,7 @@ framefb_status prepare(const Chunk& ch, int32_t ops, Prepared& P) {
     P.red->stride = A.stride;
     auto cta_of = [&](int64_t u) { return static_cast<int32_t>(((u + 1) * P.grid - 1) / units); };
     for (int j = 0; j < nm; ++j) {
-      fr::ReduceMat& R = P.red->m[j];
+      fp::ReduceMat& R = P.red->m[j];
       R.dC = ch.mats[j]->dC;
       R.nnz = header_of(ch.mats[j]->plan)->nnz;
       R.seff = A.m[j].seff;
@@ -291,7 +294,7 @@ framefb_status prepare(const Chunk& ch, int32_t ops, Prepared& P) {
 // Launch parameters live on the heap: too large for the stack of some callers.
 struct Buffers {
   std::unique_ptr<fr::Launch> a{new fr::Launch};
-  std::unique_ptr<fr::Reduce> r{new fr::Reduce};
+  std::unique_ptr<fp::Reduce> r{new fp::Reduce};
   Prepared prep() {
     Prepared p{};
     p.args = a.get();
@@ -356,8 +359,8 @@ framefb_status row_run(const framefb_mat* mats, int32_t nmats, int32_t ops, fram
         return FRAMEFB_ECUDA;
       if ((ops & FRAMEFB_OP_GRAD_COEFF) && P.nnz_max > 0) {
         void* rargs[] = {P.red};
-        if (cudaLaunchKernel(reinterpret_cast<void*>(fr::row_reduce_kernel),
-                             dim3((P.nnz_max + 31) / 32, static_cast<unsigned>(c.mats.size())), dim3(32 * fr::kLanes), rargs,
+        if (cudaLaunchKernel(reinterpret_cast<void*>(fp::pair_reduce_kernel),
+                             dim3((P.nnz_max + 31) / 32, static_cast<unsigned>(c.mats.size())), dim3(32 * fp::kLanes), rargs,
                              0, st) != cudaSuccess)
           return FRAMEFB_ECUDA;
       }

@@ -15,10 +15,7 @@
 //               plan columns in registers, H threads per column;
 //   synthesis   Stockham passes over RZ / RG, the last one adds into the rows
 //               of Y / dX (prefetched to L2 before the SpMM).
-// Every value is a token pair: complex element i of a buffer is the float4
-// (re t0, re t1, im t0, im t1), so one fp32x2 instruction serves both tokens,
-// a coefficient (frame column 2i + s) is one float2, and the SpMM gathers
-// both tokens with one 8-byte access.
+// (Token pairs: framefb_pair.cuh.)
 //
 // Bound: shared memory.  At d = 4096 a token pair moves about 13 k wavefronts
 // (four transforms of four passes and the SpMM's gathers), against 9 k issue
@@ -32,19 +29,18 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
-#include "framefb_ptx.cuh"
-#include "plan_layout.h"
+#include "framefb_pair.cuh"
 
 namespace ffb {
 namespace row {
 
+using namespace pair;
+
 // Bounded waits of the row kernel that gave up (see framefb_wait_timeouts).
 __device__ unsigned int g_row_timeouts;
 
-enum { kF = 1, kD = 2, kC = 4 };
 constexpr int kMaxShapes = 8;   // distinct geometries of a launch
 constexpr int kMaxMats = 96;    // matrices of a launch
-constexpr int kColumns = 256;   // plan columns (FRAMEFB_THREADS)
 
 // Passes of a DFT_K: radix of pass q, product of the earlier radices (a power
 // of two: an odd factor comes last), passes.
@@ -129,79 +125,14 @@ struct Launch {
   Mat m[kMaxMats];
 };
 
-// ---------------------------------------------------------------------------
-// token-pair arithmetic
-// ---------------------------------------------------------------------------
-using f2 = uint64_t;
-struct C2 {
-  f2 re, im;
-};
-
-__device__ __forceinline__ f2 pk(float a, float b) {
-  f2 r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-  return r;
-}
-__device__ __forceinline__ void unpk(f2 x, float& a, float& b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(x)); }
-__device__ __forceinline__ f2 add2(f2 a, f2 b) {
-  f2 r;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ f2 sub2(f2 a, f2 b) {
-  f2 r;
-  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ f2 mul2(f2 a, f2 b) {
-  f2 r;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) {
-  f2 r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-  return r;
-}
-__device__ __forceinline__ C2 cadd(C2 a, C2 b) { return C2{add2(a.re, b.re), add2(a.im, b.im)}; }
-__device__ __forceinline__ C2 csub(C2 a, C2 b) { return C2{sub2(a.re, b.re), sub2(a.im, b.im)}; }
-// x * w, w = (c c, s s)
-__device__ __forceinline__ C2 cmul(C2 x, C2 w) {
-  return C2{sub2(mul2(x.re, w.re), mul2(x.im, w.im)), fma2(x.im, w.re, mul2(x.re, w.im))};
-}
-// a + i S b, S = +1 or -1
-template <int S>
-__device__ __forceinline__ C2 addi(C2 a, C2 b) {
-  return S > 0 ? C2{sub2(a.re, b.im), add2(a.im, b.re)} : C2{add2(a.re, b.im), sub2(a.im, b.re)};
-}
-
 // DFT of R values in place, natural order: X_q = sum_r x_r e^{S 2 pi i q r / R}
 template <int R, int S>
 struct Dft;
 
 template <int S>
-__device__ __forceinline__ void dft4(C2& a, C2& b, C2& c, C2& d) {
-  const C2 t0 = cadd(a, c), t1 = csub(a, c), t2 = cadd(b, d), t3 = csub(b, d);
-  a = cadd(t0, t2);
-  c = csub(t0, t2);
-  b = addi<S>(t1, t3);
-  d = addi<-S>(t1, t3);
-}
-template <int S>
 struct Dft<4, S> {
   static __device__ __forceinline__ void run(C2 (&x)[4]) { dft4<S>(x[0], x[1], x[2], x[3]); }
 };
-
-// x * e^{S 2 pi i q / 8}, q = 1 or 3
-template <int S, int Q>
-__device__ __forceinline__ C2 rot8(C2 x) {
-  const f2 h = pk(0.70710678118654752f, 0.70710678118654752f), nh = pk(-0.70710678118654752f, -0.70710678118654752f);
-  if (Q == 1)  // (1 + i S) / sqrt 2
-    return S > 0 ? C2{mul2(sub2(x.re, x.im), h), mul2(add2(x.re, x.im), h)}
-                 : C2{mul2(add2(x.re, x.im), h), mul2(sub2(x.im, x.re), h)};
-  return S > 0 ? C2{mul2(add2(x.re, x.im), nh), mul2(sub2(x.re, x.im), h)}  // (-1 + i S) / sqrt 2
-               : C2{mul2(sub2(x.im, x.re), h), mul2(add2(x.re, x.im), nh)};
-}
 
 template <int S>
 struct Dft<8, S> {
@@ -301,12 +232,6 @@ __device__ __forceinline__ float w_im(W w) { return __uint_as_float(w & 0xFFFF00
 __device__ __forceinline__ W w_axpy(W y, float s, float a, float b) {
   return pack_bf16(fmaf(s, a, w_re(y)), fmaf(s, b, w_im(y)));
 }
-
-__device__ __forceinline__ C2 lds_c(const float4* p) {
-  const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(p);
-  return C2{v.x, v.y};
-}
-__device__ __forceinline__ void sts_c(float4* p, C2 x) { *reinterpret_cast<ulonglong2*>(p) = make_ulonglong2(x.re, x.im); }
 
 // The current matrix, in shared memory.
 struct Cur {
@@ -445,93 +370,6 @@ __device__ __forceinline__ void pass_k(int k, int q, const Cur& cur, int oPairs,
   }
 }
 
-// This thread's share of a plan column: KE entries of each path.
-// zw: V slot | RZ store slot << 16; gw: U slot | RG store slot << 16.
-// zcarry / gcarry: where the run that the column's first half leaves open is
-// stored by the second half (FFB_NO_STORE: none).  The coefficient values of
-// both paths and the V slots of the column path are registers for KE = 4; for
-// KE = 8 they sit in shared memory (three arrays of one float4 per four
-// entries and thread): with all six arrays in registers the transforms'
-// registers spilled to local memory, and those loads bounded the kernel.
-template <int KE>
-struct Share {
-  static constexpr bool kSm = KE > 4;
-  uint32_t zw[KE], gw[KE];
-  uint32_t gb[kSm ? 1 : KE];
-  float zc[kSm ? 1 : KE], gc[kSm ? 1 : KE];
-  uint32_t zcarry, gcarry;
-  int hZ, hG;
-};
-__host__ __device__ constexpr int plan_bytes(int NT, int KE) { return KE > 4 ? 3 * KE * NT * 4 : 0; }
-
-// entries i0 .. i0 + 3 of array a (0 zc, 1 gc, 2 gb) of this thread
-template <int KE, int NT>
-__device__ __forceinline__ void get_plan(const uint8_t* sp, int a, int i0, uint32_t (&v)[4]) {
-  const uint4 x = reinterpret_cast<const uint4*>(sp)[(a * (KE / 4) + i0 / 4) * NT + threadIdx.x];
-  v[0] = x.x;
-  v[1] = x.y;
-  v[2] = x.z;
-  v[3] = x.w;
-}
-
-template <int KE, int H, int NT>
-__device__ __forceinline__ void load_share(Share<KE>& ch, uint8_t* sp, int mode, const uint8_t* plan, const float* c_val,
-                                           int col, int half) {
-  const bool F = mode & kF, D = mode & kD, C = mode & kC;
-  const FfbPlanHeader& h = *reinterpret_cast<const FfbPlanHeader*>(plan);
-  auto tab = [&](int32_t off) { return reinterpret_cast<const int32_t*>(plan + off); };
-  ch.hZ = F ? (h.EZ + H - 1) / H : 0;
-  ch.hG = D || C ? (h.EG + H - 1) / H : 0;
-  bool openZ = false, openG = false;  // the last entry of the share continues
-  uint32_t firstZ = FFB_NO_STORE, firstG = FFB_NO_STORE;
-  auto put = [&](int a, int i, uint32_t x) {
-    reinterpret_cast<uint32_t*>(sp)[((a * (KE / 4) + i / 4) * NT + threadIdx.x) * 4 + (i & 3)] = x;
-  };
-#pragma unroll
-  for (int i = 0; i < KE; ++i) {
-    uint32_t zw = FFB_NO_STORE << 16, gw = FFB_NO_STORE << 16, gb = 0;
-    float zc = 0.f, gc = 0.f;
-    const int ez = half * ch.hZ + i, eg = half * ch.hG + i;
-    if (i < ch.hZ && ez < h.EZ) {
-      zw = static_cast<uint32_t>(__ldg(tab(h.off_zb) + ez * kColumns + col)) & ~0x8000u;
-      const int32_t qi = __ldg(tab(h.off_zq) + ez * kColumns + col);
-      zc = qi >= 0 ? __ldg(c_val + qi) : 0.f;
-      const uint32_t tg = zw >> 16;
-      openZ = qi >= 0 && tg == FFB_NO_STORE;
-      if (firstZ == FFB_NO_STORE) firstZ = tg;
-    }
-    if (i < ch.hG && eg < h.EG) {
-      gw = static_cast<uint32_t>(__ldg(tab(h.off_ga) + eg * kColumns + col)) & ~0x8000u;
-      gb = static_cast<uint32_t>(__ldg(tab(h.off_gb) + eg * kColumns + col));
-      const int32_t qi = __ldg(tab(h.off_gq) + eg * kColumns + col);
-      gc = (D && qi >= 0) ? __ldg(c_val + qi) : 0.f;
-      const uint32_t tg = gw >> 16;
-      openG = qi >= 0 && tg == FFB_NO_STORE;
-      if (!D) gw |= FFB_NO_STORE << 16;
-      if (firstG == FFB_NO_STORE) firstG = tg;
-    }
-    ch.zw[i] = zw;
-    ch.gw[i] = gw;
-    if constexpr (Share<KE>::kSm) {
-      put(0, i, __float_as_uint(zc));
-      put(1, i, __float_as_uint(gc));
-      put(2, i, gb);
-    } else {
-      ch.zc[i] = zc;
-      ch.gc[i] = gc;
-      ch.gb[i] = gb;
-    }
-  }
-  ch.zcarry = ch.gcarry = FFB_NO_STORE;
-  if constexpr (H == 2) {
-    const uint32_t open = __shfl_xor_sync(0xffffffffu, (openZ ? 1u : 0u) | (openG ? 2u : 0u), 16);
-    if (half == 1) {
-      if (open & 1u) ch.zcarry = firstZ;
-      if ((open & 2u) && D) ch.gcarry = firstG;
-    }
-  }
-}
-
 // ---------------------------------------------------------------------------
 // NT threads: H = NT / 256 threads per plan column (the two halves of a
 // column sit 16 lanes apart, so that the half-warps of a gather are the same
@@ -564,6 +402,7 @@ __global__ void __launch_bounds__(NT, NT == 512 ? 1 : 2) row_kernel(const __grid
   }
   __syncthreads();
 
+  auto slot = [](int, uint32_t x) { return x; };  // buffers in the order of the frame columns
   auto next_mat = [&](int j, int64_t u) {
     while (u >= args.m[j].ubeg + args.m[j].ntiles) ++j;
     return j;
@@ -590,7 +429,7 @@ __global__ void __launch_bounds__(NT, NT == 512 ? 1 : 2) row_kernel(const __grid
   int j = next_mat(0, u_begin);
   if (tid == 0) issue(j, u_begin);
 
-  Share<KE> ch;
+  Share<KE> ch{};
   float dc[KE];
   int cur = -1, cur_shape = -1, nfZ = 0, nfix = 0;
   int k0 = 0, k1 = 0, PP = 1;
@@ -599,18 +438,7 @@ __global__ void __launch_bounds__(NT, NT == 512 ? 1 : 2) row_kernel(const __grid
   bool failed = false;
 
   auto flush = [&](int mat) {  // dC partial sums of this thread's entries to the CTA's slot of the matrix
-    if (!C) return;
-    const FfbPlanHeader& h = *reinterpret_cast<const FfbPlanHeader*>(plan);
-    const int32_t* gq = reinterpret_cast<const int32_t*>(plan + h.off_gq);
-    float* dst = args.partial + static_cast<size_t>(blockIdx.x + mat) * args.stride;
-#pragma unroll
-    for (int i = 0; i < KE; ++i) {
-      const int e = half * ch.hG + i;
-      if (i < ch.hG && e < h.EG) {
-        const int32_t qi = __ldg(gq + e * kColumns + col);
-        if (qi >= 0) dst[qi] = dc[i];
-      }
-    }
+    if (C) flush_dc(plan, args.partial + static_cast<size_t>(blockIdx.x + mat) * args.stride, dc, ch.hG, col, half);
   };
 
   // Barrier between passes.  With a side per half of the CTA the sides share
@@ -636,7 +464,7 @@ __global__ void __launch_bounds__(NT, NT == 512 ? 1 : 2) row_kernel(const __grid
       const FfbPlanHeader& h = *reinterpret_cast<const FfbPlanHeader*>(plan);
       nfZ = F ? h.nfixZ : 0;
       nfix = nfZ + (D ? h.nfixG : 0);
-      load_share<KE, H, NT>(ch, smem + args.oPlan, mode, plan, M.c_val, col, half);
+      load_share<KE, H, NT>(ch, smem + args.oPlan, mode, plan, M.c_val, col, half, slot);
 #pragma unroll
       for (int i = 0; i < KE; ++i) dc[i] = 0.f;
       if (tid < 2) {
@@ -711,109 +539,13 @@ __global__ void __launch_bounds__(NT, NT == 512 ? 1 : 2) row_kernel(const __grid
     // ---- coefficient SpMM
     for (int p = 0; p < npair; ++p) {
       float2* base = pairs + p * cur_s.pair;
-      const float2* V = base + cur_s.A[0];
-      const float2* U = base + cur_s.A[1];
-      float2* RG = base + cur_s.B[0];
-      float2* RZ = base + cur_s.B[1];
-      if (D || C) {
-        float2 acc = make_float2(0.f, 0.f);
-#pragma unroll
-        for (int i0 = 0; i0 < KE; i0 += 4) {  // four entries' gathers in flight
-          if (i0 >= ch.hG) continue;
-          float2 ub[4], vb[4];
-          uint32_t gb[4], gc[4];
-          if constexpr (Share<KE>::kSm) {
-            get_plan<KE, NT>(smem + args.oPlan, 2, i0, gb);
-            get_plan<KE, NT>(smem + args.oPlan, 1, i0, gc);
-          } else {
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              gb[e] = ch.gb[e];
-              gc[e] = __float_as_uint(ch.gc[e]);
-            }
-          }
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            ub[e] = U[ch.gw[i0 + e] & 0xFFFFu];
-            vb[e] = C ? V[gb[e]] : make_float2(0.f, 0.f);
-          }
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            dc[i0 + e] = fmaf(ub[e].x, vb[e].x, fmaf(ub[e].y, vb[e].y, dc[i0 + e]));
-            const float c = __uint_as_float(gc[e]);
-            acc.x = fmaf(c, ub[e].x, acc.x);
-            acc.y = fmaf(c, ub[e].y, acc.y);
-            const uint32_t tg = ch.gw[i0 + e] >> 16;
-            if (tg != FFB_NO_STORE) {
-              RG[tg] = acc;
-              acc = make_float2(0.f, 0.f);
-            }
-          }
-        }
-        if constexpr (H == 2) {
-          const float cx = __shfl_xor_sync(0xffffffffu, acc.x, 16), cy = __shfl_xor_sync(0xffffffffu, acc.y, 16);
-          if (ch.gcarry != FFB_NO_STORE) {
-            const float2 o = RG[ch.gcarry];
-            RG[ch.gcarry] = make_float2(cx + o.x, cy + o.y);
-          }
-        }
-      }
-      if (F) {
-        float2 acc = make_float2(0.f, 0.f);
-#pragma unroll
-        for (int i0 = 0; i0 < KE; i0 += 4) {
-          if (i0 >= ch.hZ) continue;
-          float2 vz[4];
-          uint32_t zc[4];
-          if constexpr (Share<KE>::kSm) {
-            get_plan<KE, NT>(smem + args.oPlan, 0, i0, zc);
-          } else {
-#pragma unroll
-            for (int e = 0; e < 4; ++e) zc[e] = __float_as_uint(ch.zc[e]);
-          }
-#pragma unroll
-          for (int e = 0; e < 4; ++e) vz[e] = V[ch.zw[i0 + e] & 0xFFFFu];
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const float c = __uint_as_float(zc[e]);
-            acc.x = fmaf(c, vz[e].x, acc.x);
-            acc.y = fmaf(c, vz[e].y, acc.y);
-            const uint32_t tg = ch.zw[i0 + e] >> 16;
-            if (tg != FFB_NO_STORE) {
-              RZ[tg] = acc;
-              acc = make_float2(0.f, 0.f);
-            }
-          }
-        }
-        if constexpr (H == 2) {
-          const float cx = __shfl_xor_sync(0xffffffffu, acc.x, 16), cy = __shfl_xor_sync(0xffffffffu, acc.y, 16);
-          if (ch.zcarry != FFB_NO_STORE) {
-            const float2 o = RZ[ch.zcarry];
-            RZ[ch.zcarry] = make_float2(cx + o.x, cy + o.y);
-          }
-        }
-      }
+      spmm<KE, H, NT>(ch, dc, smem + args.oPlan, F, D, C, base + cur_s.A[0], base + cur_s.A[1], base + cur_s.B[0],
+                      base + cur_s.B[1]);
     }
     __syncthreads();
     if (kSyn) {
       if (nfix > 0) {
-        // rows (columns) split between plan columns: add the overflow pieces
-        const FfbPlanHeader& h = *reinterpret_cast<const FfbPlanHeader*>(plan);
-        const int4* fz = reinterpret_cast<const int4*>(plan + h.off_fixZ);
-        const int4* fg = reinterpret_cast<const int4*>(plan + h.off_fixG);
-        for (int w = tid; w < nfix * npair; w += NT) {
-          const int p = w / nfix, i = w - p * nfix;
-          const bool z = i < nfZ;
-          const int4 it = z ? __ldg(fz + i) : __ldg(fg + (i - nfZ));
-          float2* R = pairs + p * cur_s.pair + cur_s.B[z ? 1 : 0];
-          float2 a = R[it.x];
-          for (int c = 0; c < it.z; ++c) {
-            const float2 o = R[it.y + c];
-            a.x += o.x;
-            a.y += o.y;
-          }
-          R[it.x] = a;
-        }
+        fix_runs<NT>(plan, nfZ, nfix, npair, pairs + cur_s.B[0], pairs + cur_s.B[1], cur_s.pair, slot);
         __syncthreads();
       }
       // ---- synthesis: both sides start together
@@ -836,39 +568,6 @@ __global__ void __launch_bounds__(NT, NT == 512 ? 1 : 2) row_kernel(const __grid
     return;
   }
   if (cur >= 0) flush(cur);
-}
-
-// dC_q = seff * sum over the CTAs that visited the matrix, in a fixed order:
-// kLanes interleaved sums, then a tree over them.
-struct ReduceMat {
-  float* dC;
-  int32_t c0, c1, nnz;  // CTAs [c0, c1] visited the matrix
-  float seff;
-};
-struct Reduce {
-  const float* partial;
-  int32_t stride, pad;
-  ReduceMat m[kMaxMats];
-};
-constexpr int kLanes = 8;
-
-__global__ void __launch_bounds__(256) row_reduce_kernel(const __grid_constant__ Reduce r) {
-  const int j = blockIdx.y;
-  const ReduceMat& M = r.m[j];
-  // lane l of a group of 8 warps' lanes: entry q = 32 x block + lane, part = warp
-  __shared__ float s[kLanes][32];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int q = blockIdx.x * 32 + lane;
-  float a = 0.f;
-  if (q < M.nnz)
-    for (int c = M.c0 + w; c <= M.c1; c += kLanes) a += r.partial[static_cast<size_t>(c + j) * r.stride + q];
-  s[w][lane] = a;
-  __syncthreads();
-  if (w == 0 && q < M.nnz) {
-    const float x = ((s[0][lane] + s[1][lane]) + (s[2][lane] + s[3][lane])) +
-                    ((s[4][lane] + s[5][lane]) + (s[6][lane] + s[7][lane]));
-    M.dC[q] = M.seff * x;
-  }
 }
 
 }  // namespace row
