@@ -993,16 +993,24 @@ extern "C" framefb_status framefb_merge(const void* W0, framefb_dtype dtype, int
   void* kargs[] = {&a};
   void* fn = dtype == FRAMEFB_BF16 ? reinterpret_cast<void*>(ffb::merge_kernel<__nv_bfloat16>)
                                    : reinterpret_cast<void*>(ffb::merge_kernel<float>);
-  // grid-stride over (out group, tenant) items: as many CTAs as are resident
   int dev = 0, sms = 0, per_sm = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, ffb::kMergeThreads, 0) != cudaSuccess)
     return FRAMEFB_ECUDA;
-  // one warp per (out group, tenant, run of blocks) item
-  const int64_t items =
-      static_cast<int64_t>(h->Gm) * T * ((h->Gn + ffb::kMergeBlocks - 1) / ffb::kMergeBlocks);
-  const int64_t grid = std::max<int64_t>(
-      1, std::min<int64_t>((items + ffb::kMergeWarps - 1) / ffb::kMergeWarps, static_cast<int64_t>(sms) * std::max(per_sm, 1)));
+  // one wave of CTAs: the tenants of an out group in as many runs as are
+  // resident, then (few tenants) its blocks in runs of at least a warp each
+  const int64_t resident = std::max<int64_t>(1, static_cast<int64_t>(sms) * std::max(per_sm, 1));
+  // (tenants go in twos: an odd run would end on a half-used pass)
+  const int64_t chunks = std::max<int64_t>(1, std::min<int64_t>((T + 1) / 2, resident / h->Gm));
+  const int64_t splits = std::max<int64_t>(
+      1, std::min<int64_t>((h->Gn + ffb::kMergeWarps - 1) / ffb::kMergeWarps, resident / (h->Gm * chunks)));
+  a.Gn = h->Gn;
+  a.Gm = h->Gm;
+  a.off_blkptr = h->off_blkptr;
+  a.off_blkent = h->off_blkent;
+  a.chunks = static_cast<int32_t>(chunks);
+  a.splits = static_cast<int32_t>(splits);
+  const int64_t grid = static_cast<int64_t>(h->Gm) * chunks * splits;
   if (cudaLaunchKernel(fn, dim3(static_cast<unsigned>(grid)), dim3(ffb::kMergeThreads), kargs, 0,
                        static_cast<cudaStream_t>(stream)) != cudaSuccess)
     return FRAMEFB_ECUDA;

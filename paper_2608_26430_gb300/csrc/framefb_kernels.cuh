@@ -19,6 +19,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 #include "framefb.h"
 #include "plan_layout.h"
 
@@ -86,6 +88,8 @@ struct MergeK {
   const float* fout_val;
   int64_t ldw;
   int32_t m, n, rho_in, rho_out, nnz, T;
+  int32_t splits, chunks;  // CTAs per out group: runs of blocks x runs of tenants
+  int32_t Gn, Gm, off_blkptr, off_blkent;  // of the plan
   float seff;
 };
 
@@ -751,17 +755,20 @@ __global__ void __launch_bounds__(256) dc_reduce_kernel(const __grid_constant__ 
 // ---------------------------------------------------------------------------
 // Merge (Sec. 3.4 "Storage efficiency", Alg. 1 step 6 per tenant):
 //   W_t[32g + i][32h + j] = W0[..] + (s/16) sum_{e in block (g,h)} c_{t,e} Dout[i][a_e] Din[j][b_e],
-// D = 4 x the group-0 block of each frame (k = 16, k*rho = d frames), staged
-// once per CTA.  Work items are (out group g, tenant t, a run of four 32 x 32
-// blocks h of that row); each warp takes items grid-stride (any number of
-// tenants).  A warp first stages its item's entries (the blocks (g, .) are
-// contiguous in the plan) and the tenant's values in its own slice of
-// shared memory, so no CTA barrier ties the warps together and one warp's
-// staging latency hides behind the others' arithmetic.  A
-// lane owns one 16-byte chunk of one row per row pass: lanes (row l / CPR,
-// chunk l % CPR), CPR = 16-byte chunks per 32-element row (4 bf16, 8 fp32),
-// so a warp's store covers whole 64- or 128-byte row segments.  Bound: HBM
-// (W_t written once; W0 and the plan are L2-resident across tenants).
+// D = 4 x the group-0 block of each frame (k = 16, k*rho = d frames).  A CTA
+// takes one out group g, a run of its 32 x 32 blocks h and a run of tenants: the
+// entries of the blocks (contiguous in the plan) and the tenants' values of them
+// are staged in shared memory once, so no global load sits in the loops.  A warp
+// takes blocks in turn and two tenants at a time: W0, the frame factors and the
+// entries are read once for both, and the products run on pairs of columns
+// (fp32x2).  A lane owns one 16-byte chunk of one row per row pass: lanes (row
+// l / CPR, chunk l % CPR), CPR = 16-byte chunks per 32-element row (4 bf16, 8
+// fp32), so a warp's store covers whole 64- or 128-byte row segments.  Bound:
+// the writes of W_t: 64 tenants of 768^2, 2000 entries, take 26.4 us in bf16
+// (75 MB) and 33 us in fp32, 19 us of the former without any entry; 8 tenants of
+// 4096^2 59 us (5.1 TB/s).  With one warp per (group, tenant, four blocks) that
+// staged its own entries the loads' latency and the factors' re-reads bounded
+// it: 30, 39.5 and 77 us.
 // ---------------------------------------------------------------------------
 template <typename Elem>
 struct MergeIO;
@@ -802,8 +809,25 @@ struct MergeIO<float> {
 
 constexpr int kMergeThreads = 256;
 constexpr int kMergeWarps = kMergeThreads / 32;
-constexpr int kMergeStage = 512;  // entries of one item a warp stages (longer rows read them from L2)
-constexpr int kMergeBlocks = 4;   // 32 x 32 blocks per work item
+constexpr int kMergeEnt = 1024;  // entries a CTA stages (longer runs of blocks read them from L2)
+constexpr int kMergeBlk = 1024;  // blocks of an out group (a plan has at most 32768 columns)
+constexpr int kMergeVal = 4096;  // staged coefficient values: tenants x entries
+
+__device__ __forceinline__ uint64_t f2_pack(float a, float b) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t f2_fma(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ uint64_t f2_mul(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
 
 template <typename Elem>
 __global__ void __launch_bounds__(kMergeThreads, 2) merge_kernel(const __grid_constant__ MergeK a) {
@@ -812,109 +836,128 @@ __global__ void __launch_bounds__(kMergeThreads, 2) merge_kernel(const __grid_co
   constexpr int CPR = 32 / PER;             // chunks per 32-element block row
   constexpr int RPP = 32 / CPR;             // rows per warp pass
   constexpr int PASSES = 32 / RPP;          // passes over the block's 32 rows
-  __shared__ float DoutT[32][33];           // [a][i] = Dout[i][a]
+  __shared__ float2 Dout2[32][33];              // [a][i] = (Dout[i][a], Dout[i][a])
   __shared__ __align__(16) float DinT[32][32];  // [b][j] = Din[j][b]
-  __shared__ int32_t ent_s[kMergeWarps][kMergeStage];  // a_local | b_local << 8, per warp
-  __shared__ float cv_s[kMergeWarps][kMergeStage];     // the tenant's value of each
-  __shared__ int32_t bp_s[kMergeWarps][kMergeBlocks + 1];  // block boundaries of the item
-  for (int idx = threadIdx.x; idx < 1024; idx += blockDim.x) {
-    const int w = idx & 31, x = idx >> 5, i = x >> 1, s = x & 1;  // column x = 2i + s of the group block, row w
-    DoutT[x][w] = 4.f * __ldg(a.fout_val + 32 * (i * a.rho_out + s) + w);
-    DinT[x][w] = 4.f * __ldg(a.fin_val + 32 * (i * a.rho_in + s) + w);
-  }
-  __syncthreads();
-  const FfbPlanHeader& h = hdr(a.plan);
-  const int32_t* blkptr = table<int32_t>(a.plan, h.off_blkptr);
-  const int2* blkent = table<int2>(a.plan, h.off_blkent);
+  __shared__ int32_t ent_s[kMergeEnt];          // a_local | b_local << 8
+  __shared__ int32_t q_s[kMergeEnt];            // index of its value
+  __shared__ float cv_s[kMergeVal];             // [tenant][entry]
+  __shared__ int32_t ptr_s[kMergeBlk + 1];      // entry ranges of the CTA's blocks (from its first entry)
+  const int2* blkent = table<int2>(a.plan, a.off_blkent);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int rl = lane / CPR, cl = lane % CPR;  // row in the pass, chunk in the row
-  int32_t* ent = ent_s[warp];
-  float* cvw = cv_s[warp];
-  int32_t* bp = bp_s[warp];
-  const Elem* W0 = static_cast<const Elem*>(a.W0);
-  // work items: (out group g, tenant t, run of kMergeBlocks blocks)
-  const int nsub = (h.Gn + kMergeBlocks - 1) / kMergeBlocks;
-  const int64_t items = static_cast<int64_t>(h.Gm) * nsub * a.T;
-  for (int64_t it = static_cast<int64_t>(blockIdx.x) * kMergeWarps + warp; it < items;
-       it += static_cast<int64_t>(gridDim.x) * kMergeWarps) {
-    const int sub = static_cast<int>(it % nsub);
-    const int g = static_cast<int>((it / nsub) % h.Gm);
-    const int64_t t = it / (static_cast<int64_t>(nsub) * h.Gm);
-    const int hb0 = sub * kMergeBlocks, hb1 = min(h.Gn, hb0 + kMergeBlocks);
-    const float* cv = a.c_vals + t * a.nnz;
-    Elem* Wt = static_cast<Elem*>(a.Wout) + t * static_cast<int64_t>(a.m) * a.ldw;
-    const int eg0 = __ldg(blkptr + g * h.Gn + hb0), eg1 = __ldg(blkptr + g * h.Gn + hb1);
-    const bool staged = eg1 - eg0 <= kMergeStage;
-    __syncwarp();  // the warp's previous item is done with its slice
-    if (staged) {
-      for (int e = lane; e < eg1 - eg0; e += 32) {
-        const int2 en = __ldg(blkent + eg0 + e);
-        ent[e] = en.x;
-        cvw[e] = __ldg(cv + en.y);
-      }
-      if (lane <= hb1 - hb0) bp[lane] = __ldg(blkptr + g * h.Gn + hb0 + lane);
+  // this CTA's out group, blocks [h0, h1) and tenants [t0, t1)
+  const int g = blockIdx.x % a.Gm, part = blockIdx.x / a.Gm;
+  const int split = part % a.splits, chunk = part / a.splits;
+  const int h0 = static_cast<int>(static_cast<int64_t>(a.Gn) * split / a.splits);
+  const int h1 = static_cast<int>(static_cast<int64_t>(a.Gn) * (split + 1) / a.splits);
+  const int64_t pairs = (static_cast<int64_t>(a.T) + 1) / 2;  // tenants go in twos
+  const int64_t t0 = 2 * (pairs * chunk / a.chunks), t1 = min(static_cast<int64_t>(a.T), 2 * (pairs * (chunk + 1) / a.chunks));
+  const int32_t* blkptr = table<int32_t>(a.plan, a.off_blkptr) + g * a.Gn + h0;
+  const int eg0 = __ldg(blkptr), ne = __ldg(blkptr + (h1 - h0)) - eg0;
+  for (int x = threadIdx.x; x <= h1 - h0; x += kMergeThreads) ptr_s[x] = __ldg(blkptr + x) - eg0;
+  const bool staged = ne <= kMergeEnt;
+  const int tb = staged ? (ne > 0 ? min(static_cast<int64_t>(kMergeVal / ne), t1 - t0) : t1 - t0) : t1 - t0;  // tenants per batch
+  if (staged) {
+    for (int e = threadIdx.x; e < ne; e += kMergeThreads) {
+      const int2 en = __ldg(blkent + eg0 + e);
+      ent_s[e] = en.x;
+      q_s[e] = en.y;
     }
-    __syncwarp();
-    // W0 chunks one block ahead: their latency overlaps the previous block
-    uint4 w0n[PASSES];
-#pragma unroll
-    for (int r = 0; r < PASSES; ++r)
-      w0n[r] = __ldg(reinterpret_cast<const uint4*>(W0 + static_cast<int64_t>(32 * g + r * RPP + rl) * a.ldw +
-                                                    32 * hb0 + cl * PER));
-    for (int hb = hb0; hb < hb1; ++hb) {
-      uint4 w0[PASSES];
-#pragma unroll
-      for (int r = 0; r < PASSES; ++r) w0[r] = w0n[r];
-      if (hb + 1 < hb1) {
-#pragma unroll
-        for (int r = 0; r < PASSES; ++r)
-          w0n[r] = __ldg(reinterpret_cast<const uint4*>(W0 + static_cast<int64_t>(32 * g + r * RPP + rl) * a.ldw +
-                                                        32 * (hb + 1) + cl * PER));
+  }
+  for (int idx = threadIdx.x; idx < 1024; idx += kMergeThreads) {
+    const int w = idx & 31, x = idx >> 5, i = x >> 1, s = x & 1;  // column x = 2i + s of the group block, row w
+    const float o = 4.f * __ldg(a.fout_val + 32 * (i * a.rho_out + s) + w);
+    Dout2[x][w] = make_float2(o, o);
+    DinT[x][w] = 4.f * __ldg(a.fin_val + 32 * (i * a.rho_in + s) + w);
+  }
+  const Elem* W0 = static_cast<const Elem*>(a.W0) + static_cast<int64_t>(32 * g + rl) * a.ldw + cl * PER;
+  const int64_t tstride = static_cast<int64_t>(a.m) * a.ldw;
+  const uint64_t seff2 = f2_pack(a.seff, a.seff);
+  for (int64_t tb0 = t0; tb0 < t1; tb0 += tb) {
+    const int nt = static_cast<int>(min(static_cast<int64_t>(tb), t1 - tb0));
+    __syncthreads();  // entries staged; the previous batch's values are no longer read
+    if (staged) {
+      for (int x = threadIdx.x; x < nt * ne; x += kMergeThreads) {
+        const int t = x / ne, e = x - t * ne;
+        cv_s[x] = __ldg(a.c_vals + (tb0 + t) * a.nnz + q_s[e]);
       }
-      float acc[PASSES][PER];
-#pragma unroll
-      for (int r = 0; r < PASSES; ++r)
-#pragma unroll
-        for (int j = 0; j < PER; ++j) acc[r][j] = 0.f;
-      const int e0 = staged ? bp[hb - hb0] : __ldg(blkptr + g * h.Gn + hb);
-      const int e1 = staged ? bp[hb - hb0 + 1] : __ldg(blkptr + g * h.Gn + hb + 1);
-      for (int e = e0; e < e1; ++e) {
-        int ex;
-        float c;
-        if (staged) {
-          ex = ent[e - eg0];
-          c = cvw[e - eg0];
-        } else {
-          const int2 en = __ldg(blkent + e);
-          ex = en.x;
-          c = __ldg(cv + en.y);
-        }
-        const int al = ex & 31, bl = (ex >> 8) & 31;
-        float din[PER];
-#pragma unroll
-        for (int j = 0; j < PER; j += 4) {
-          const float4 q = *reinterpret_cast<const float4*>(&DinT[bl][cl * PER + j]);
-          din[j] = q.x;
-          din[j + 1] = q.y;
-          din[j + 2] = q.z;
-          din[j + 3] = q.w;
-        }
-#pragma unroll
-        for (int r = 0; r < PASSES; ++r) {
-          const float u = c * DoutT[al][r * RPP + rl];
-#pragma unroll
-          for (int j = 0; j < PER; ++j) acc[r][j] = fmaf(u, din[j], acc[r][j]);
-        }
-      }
+    }
+    __syncthreads();
+    for (int hb = h0 + warp; hb < h1; hb += kMergeWarps) {
+      const int e0 = ptr_s[hb - h0], e1 = ptr_s[hb - h0 + 1];
+      uint64_t w0[PASSES][PER / 2];
 #pragma unroll
       for (int r = 0; r < PASSES; ++r) {
-        const int64_t off = static_cast<int64_t>(32 * g + r * RPP + rl) * a.ldw + 32 * hb + cl * PER;
         float w[PER];
-        IO::unpack(w0[r], w);
+        IO::unpack(__ldg(reinterpret_cast<const uint4*>(W0 + static_cast<int64_t>(r * RPP) * a.ldw + 32 * hb)), w);
 #pragma unroll
-        for (int j = 0; j < PER; ++j) w[j] = fmaf(a.seff, acc[r][j], w[j]);
-        *reinterpret_cast<uint4*>(Wt + off) = IO::pack(w);
+        for (int j = 0; j < PER / 2; ++j) w0[r][j] = f2_pack(w[2 * j], w[2 * j + 1]);
       }
+      // TT tenants from batch tenant t on
+      auto tenants = [&](auto tt, int t) {
+        constexpr int TT = decltype(tt)::value;
+        uint64_t acc[TT][PASSES][PER / 2];
+#pragma unroll
+        for (int k = 0; k < TT; ++k)
+#pragma unroll
+          for (int r = 0; r < PASSES; ++r)
+#pragma unroll
+            for (int j = 0; j < PER / 2; ++j) acc[k][r][j] = 0ull;
+        for (int e = e0; e < e1; ++e) {
+          int ex;
+          float c[TT];
+          if (staged) {
+            ex = ent_s[e];
+#pragma unroll
+            for (int k = 0; k < TT; ++k) c[k] = cv_s[(t + k) * ne + e];
+          } else {
+            const int2 en = __ldg(blkent + eg0 + e);
+            ex = en.x;
+#pragma unroll
+            for (int k = 0; k < TT; ++k) c[k] = __ldg(a.c_vals + (tb0 + t + k) * a.nnz + en.y);
+          }
+          const int al = ex & 31, bl = (ex >> 8) & 31;
+          uint64_t din[PER / 2];
+#pragma unroll
+          for (int j = 0; j < PER / 2; j += 2) {
+            const ulonglong2 q = *reinterpret_cast<const ulonglong2*>(&DinT[bl][cl * PER + 2 * j]);
+            din[j] = q.x;
+            din[j + 1] = q.y;
+          }
+          uint64_t u[PASSES];
+#pragma unroll
+          for (int r = 0; r < PASSES; ++r) u[r] = *reinterpret_cast<const uint64_t*>(&Dout2[al][r * RPP + rl]);
+#pragma unroll
+          for (int k = 0; k < TT; ++k) {
+            const uint64_t cc = f2_pack(c[k], c[k]);
+#pragma unroll
+            for (int j = 0; j < PER / 2; ++j) {
+              const uint64_t cd = f2_mul(cc, din[j]);
+#pragma unroll
+              for (int r = 0; r < PASSES; ++r) acc[k][r][j] = f2_fma(u[r], cd, acc[k][r][j]);
+            }
+          }
+        }
+#pragma unroll
+        for (int k = 0; k < TT; ++k) {
+          Elem* Wt = static_cast<Elem*>(a.Wout) + (tb0 + t + k) * tstride + static_cast<int64_t>(32 * g + rl) * a.ldw +
+                     cl * PER + 32 * hb;
+#pragma unroll
+          for (int r = 0; r < PASSES; ++r) {
+            float w[PER];
+#pragma unroll
+            for (int j = 0; j < PER / 2; ++j) {
+              const uint64_t x = f2_fma(seff2, acc[k][r][j], w0[r][j]);
+              asm("mov.b64 {%0, %1}, %2;" : "=f"(w[2 * j]), "=f"(w[2 * j + 1]) : "l"(x));
+            }
+            // (written once, not read here: streaming stores leave L2 sooner, fp32 39 -> 33 us)
+            __stcs(reinterpret_cast<uint4*>(Wt + static_cast<int64_t>(r * RPP) * a.ldw), IO::pack(w));
+          }
+        }
+      };
+      int t = 0;
+      for (; t + 2 <= nt; t += 2) tenants(std::integral_constant<int, 2>{}, t);
+      if (t < nt) tenants(std::integral_constant<int, 1>{}, t);
     }
   }
 }
