@@ -15,6 +15,7 @@
 #include "framefb_dense.h"
 #include "framefb_grp.h"
 #include "framefb_kernels.cuh"
+#include "framefb_launch.h"
 #include "framefb_mma.cuh"
 #include "framefb_row.h"
 #include "framefb_tc.cuh"
@@ -675,7 +676,7 @@ framefb_status structured_run(const framefb_mat* mats, int32_t nmats, int32_t op
                : P.tc  ? tc_kernel_ptr(ops)
                        : tile_kernel_ptr(dtype, ops, P.reg, P.T);
     void* kargs[] = {(P.tc || P.tc2) ? static_cast<void*>(P.tcargs) : static_cast<void*>(P.args)};
-    if (cudaLaunchKernel(fn, dim3(P.grid), dim3(P.threads), kargs, P.smem, st) != cudaSuccess)
+    if (ffb_host::launch_chained(fn, dim3(P.grid), dim3(P.threads), kargs, P.smem, st) != cudaSuccess)
       return FRAMEFB_ECUDA;
     if (ops & FRAMEFB_OP_GRAD_COEFF) {
       int nnz_max = 0;
@@ -683,7 +684,7 @@ framefb_status structured_run(const framefb_mat* mats, int32_t nmats, int32_t op
       if (nnz_max > 0) {
         void* rargs[] = {P.red};
         const dim3 rg((nnz_max + 255) / 256, nm);
-        if (cudaLaunchKernel(reinterpret_cast<void*>(ffb::dc_reduce_kernel), rg, dim3(256), rargs, 0, st) !=
+        if (ffb_host::launch_chained(reinterpret_cast<void*>(ffb::dc_reduce_kernel), rg, dim3(256), rargs, 0, st) !=
             cudaSuccess)
           return FRAMEFB_ECUDA;
       }
@@ -1011,7 +1012,7 @@ extern "C" framefb_status framefb_merge(const void* W0, framefb_dtype dtype, int
   a.chunks = static_cast<int32_t>(chunks);
   a.splits = static_cast<int32_t>(splits);
   const int64_t grid = static_cast<int64_t>(h->Gm) * chunks * splits;
-  if (cudaLaunchKernel(fn, dim3(static_cast<unsigned>(grid)), dim3(ffb::kMergeThreads), kargs, 0,
+  if (ffb_host::launch_chained(fn, dim3(static_cast<unsigned>(grid)), dim3(ffb::kMergeThreads), kargs, 0,
                        static_cast<cudaStream_t>(stream)) != cudaSuccess)
     return FRAMEFB_ECUDA;
   return FRAMEFB_OK;
@@ -1109,7 +1110,7 @@ extern "C" framefb_status framefb_adamw(float* param, const float* grad, float* 
   const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>((work + 255) / 256, static_cast<int64_t>(sms) * 8));
   void* kargs[] = {&a};
   void* fn = vec ? reinterpret_cast<void*>(ffb::adamw_kernel<true>) : reinterpret_cast<void*>(ffb::adamw_kernel<false>);
-  if (cudaLaunchKernel(fn, dim3(static_cast<unsigned>(blocks)), dim3(256), kargs, 0, static_cast<cudaStream_t>(stream)) !=
+  if (ffb_host::launch_chained(fn, dim3(static_cast<unsigned>(blocks)), dim3(256), kargs, 0, static_cast<cudaStream_t>(stream)) !=
       cudaSuccess)
     return FRAMEFB_ECUDA;
   return FRAMEFB_OK;

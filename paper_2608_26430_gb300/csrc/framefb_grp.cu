@@ -14,6 +14,7 @@
 #include "framefb.h"
 #include "framefb_grp.cuh"
 #include "framefb_grp.h"
+#include "framefb_launch.h"
 #include "plan_internal.h"
 #include "plan_layout.h"
 
@@ -379,11 +380,11 @@ framefb_status grp_run(const framefb_mat* mats, int32_t nmats, int32_t ops, fram
       P.args->partial = static_cast<float*>(ws);
       P.red->partial = static_cast<const float*>(ws);
       void* kargs[] = {P.args};
-      if (cudaLaunchKernel(kernel_ptr(P.v, dt), dim3(P.grid), dim3(P.v.nt), kargs, P.smem, st) != cudaSuccess)
+      if (launch_chained(kernel_ptr(P.v, dt), dim3(P.grid), dim3(P.v.nt), kargs, P.smem, st) != cudaSuccess)
         return FRAMEFB_ECUDA;
       if ((ops & FRAMEFB_OP_GRAD_COEFF) && P.nnz_max > 0) {
         void* rargs[] = {P.red};
-        if (cudaLaunchKernel(reinterpret_cast<void*>(fp::pair_reduce_kernel),
+        if (launch_chained(reinterpret_cast<void*>(fp::pair_reduce_kernel),
                              dim3((P.nnz_max + 31) / 32, static_cast<unsigned>(c.mats.size())), dim3(32 * fp::kLanes), rargs,
                              0, st) != cudaSuccess)
           return FRAMEFB_ECUDA;

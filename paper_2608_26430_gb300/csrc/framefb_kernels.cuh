@@ -22,6 +22,7 @@
 #include <type_traits>
 
 #include "framefb.h"
+#include "framefb_ptx.cuh"
 #include "plan_layout.h"
 
 namespace ffb {
@@ -608,6 +609,7 @@ __device__ __forceinline__ int fix_count(const uint8_t* plan, int mode) {
 // ---------------------------------------------------------------------------
 template <int MODE, bool REG>
 __global__ void __launch_bounds__(kThreads, 1) fft_tile_kernel(const __grid_constant__ LaunchK args) {
+  chain_wait();
   using Elem = float;
   constexpr bool F = MODE & MODE_F, D = MODE & MODE_D, C = MODE & MODE_C;
   constexpr bool NEED_V = F || C, NEED_U = D || C;
@@ -738,6 +740,8 @@ __global__ void __launch_bounds__(kThreads, 1) fft_tile_kernel(const __grid_cons
 // dC_q = (s/16) * sum over the CTAs that visited the matrix, in CTA order
 // (a plan's part: q over its entries' indices).
 __global__ void __launch_bounds__(256) dc_reduce_kernel(const __grid_constant__ ReduceK r) {
+  chain_wait();
+  chain_next();
   const int j = blockIdx.y;
   const ReduceMat& M = r.m[j];
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -831,6 +835,8 @@ __device__ __forceinline__ uint64_t f2_mul(uint64_t a, uint64_t b) {
 
 template <typename Elem>
 __global__ void __launch_bounds__(kMergeThreads, 2) merge_kernel(const __grid_constant__ MergeK a) {
+  chain_wait();
+  chain_next();
   using IO = MergeIO<Elem>;
   constexpr int PER = IO::kPer;             // elements per lane chunk
   constexpr int CPR = 32 / PER;             // chunks per 32-element block row
@@ -989,6 +995,8 @@ __device__ __forceinline__ void adamw_one(float& p, float g, float& m, float& v,
 
 template <bool VEC>
 __global__ void __launch_bounds__(256) adamw_kernel(const AdamWK a) {
+  chain_wait();
+  chain_next();
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
   const int64_t i0 = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
   if constexpr (VEC) {

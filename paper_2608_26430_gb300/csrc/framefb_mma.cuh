@@ -372,6 +372,7 @@ __device__ __forceinline__ int matrix_of(const Args& args, int j, int64_t u) {
 // ---------------------------------------------------------------------------
 template <int MODE, bool REG, int T>
 __global__ void __launch_bounds__(kThreads, 1) mma_tile_kernel(const __grid_constant__ LaunchK args) {
+  chain_wait();
   static_assert(T == 1 || T == 2, "tile of one or two tokens");
   constexpr bool F = MODE & MODE_F, D = MODE & MODE_D, C = MODE & MODE_C;
   constexpr bool NEED_V = F || C, NEED_U = D || C, SYN = F || D;

@@ -341,6 +341,8 @@ struct Reduce {
 constexpr int kLanes = 8;
 
 static __global__ void __launch_bounds__(256) pair_reduce_kernel(const __grid_constant__ Reduce r) {
+  chain_wait();
+  chain_next();
   const int j = blockIdx.y;
   const ReduceMat& M = r.m[j];
   // lane l of a group of 8 warps' lanes: entry q = 32 x block + lane, part = warp

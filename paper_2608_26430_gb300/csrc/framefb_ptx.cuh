@@ -144,4 +144,12 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
   for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+// Start of a kernel launched by launch_chained (framefb_launch.h): waits until
+// the kernels ahead on the stream have ended and their writes are visible.
+// First statement of such a kernel: nothing reads or writes memory before it.
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// Lets the next kernel of the stream become resident (it waits in chain_wait)
+// once every CTA of this one has come here or ended.
+__device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 }  // namespace ffb

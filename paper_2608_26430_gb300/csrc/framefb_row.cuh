@@ -378,6 +378,8 @@ __device__ __forceinline__ void pass_k(int k, int q, const Cur& cur, int oPairs,
 // K: the DFT size of both sides of every matrix of the launch, or 0 for any.
 template <int NT, int KE, int K>
 __global__ void __launch_bounds__(NT, NT == 512 ? 1 : 2) row_kernel(const __grid_constant__ Launch args) {
+  chain_wait();
+  chain_next();
   constexpr int H = NT / kColumns;
   extern __shared__ __align__(128) uint8_t smem[];
   __shared__ Cur cur_s;

@@ -342,6 +342,7 @@ struct TileTrack {
 
 template <int MODE>
 __global__ void __launch_bounds__(kTcThreads, 1) tc_tile_kernel(const __grid_constant__ TcLaunchK args) {
+  chain_wait();
   constexpr bool F = MODE & MODE_F, D = MODE & MODE_D, C = MODE & MODE_C;
   constexpr bool NEED_V = F || C, NEED_U = D || C, SYN = F || D;
   extern __shared__ __align__(1024) uint8_t smem[];

@@ -170,6 +170,7 @@ __device__ __forceinline__ void put4(float* base, uint32_t bytes, float x) {
 // follow the segments and the coefficient values are the unit's tenant's.
 template <int MODE, bool SEG = false>
 __global__ void __launch_bounds__(kTcThreads, 1) tc2_tile_kernel(const __grid_constant__ TcLaunchK args) {
+  chain_wait();
   constexpr bool F = MODE & MODE_F, D = MODE & MODE_D, C = MODE & MODE_C;
   static_assert(!SEG || MODE == MODE_F, "segment tables serve the forward pass");
   using Track = std::conditional_t<SEG, SegTrack, TileTrack>;
