@@ -5,8 +5,10 @@
 
 #include <algorithm>
 #include <cmath>
+#include <cstddef>
 #include <cstdlib>
 #include <cstring>
+#include <memory>
 #include <mutex>
 #include <string>
 #include <vector>
@@ -345,8 +347,9 @@ framefb_status prepare(const framefb_mat* mats, int32_t nmats, int32_t ops, fram
                        const SegTable* seg = nullptr) {
   const size_t esz = dt == FRAMEFB_BF16 ? 2 : 4;
   const bool F = ops & FRAMEFB_OP_FORWARD, D = ops & FRAMEFB_OP_BACKWARD_DX, C = ops & FRAMEFB_OP_GRAD_COEFF;
-  std::memset(P.args, 0, sizeof(ffb::LaunchK));
-  std::memset(P.red, 0, sizeof(ffb::ReduceK));
+  // (the matrices' entries are filled below, the rest is never read)
+  std::memset(P.args, 0, offsetof(ffb::LaunchK, m));
+  std::memset(P.red, 0, offsetof(ffb::ReduceK, m));
   bool reg = true;
   int32_t nnz_max = 0;
   for (int32_t j = 0; j < nmats; ++j) {
@@ -387,7 +390,7 @@ framefb_status prepare(const framefb_mat* mats, int32_t nmats, int32_t ops, fram
     if (need > 0 && need <= budget) {
       tc2 = true;
       T_mma = 2;
-      std::memset(P.tcargs, 0, sizeof(ffb::TcLaunchK));
+      std::memset(P.tcargs, 0, offsetof(ffb::TcLaunchK, m));
       smem = tc2_smem_map(mats, nmats, ops, 2, pairs, pack, P.tcargs);
     }
   }
@@ -405,7 +408,7 @@ framefb_status prepare(const framefb_mat* mats, int32_t nmats, int32_t ops, fram
       if (need > 0 && need <= budget) {
         tc = true;
         T_mma = 1;
-        std::memset(P.tcargs, 0, sizeof(ffb::TcLaunchK));
+        std::memset(P.tcargs, 0, offsetof(ffb::TcLaunchK, m));
         smem = tc_smem_map(mats, nmats, ops, S, P.tcargs);
       }
     }
@@ -515,6 +518,7 @@ framefb_status prepare(const framefb_mat* mats, int32_t nmats, int32_t ops, fram
   if (tc || tc2) {
     ffb::TcLaunchK& A = *P.tcargs;
     A.nmats = nmats;
+    if (!seg) A.nseg = 0;
     A.total_units = P.args->total_units;
     A.stride = P.args->stride;
     for (int32_t j = 0; j < nmats; ++j) {
@@ -559,17 +563,23 @@ framefb_status prepare(const framefb_mat* mats, int32_t nmats, int32_t ops, fram
 }
 
 struct Buffers {
-  std::vector<uint8_t> a, t, r;
-  Buffers() : a(sizeof(ffb::LaunchK)), t(sizeof(ffb::TcLaunchK) + 64), r(sizeof(ffb::ReduceK)) {}
+  std::unique_ptr<ffb::LaunchK> a{new ffb::LaunchK};
+  std::unique_ptr<ffb::TcLaunchK> t{new ffb::TcLaunchK};  // (aligned for its tensor maps)
+  std::unique_ptr<ffb::ReduceK> r{new ffb::ReduceK};
   Prepared prep() {
     Prepared p{};
-    p.args = reinterpret_cast<ffb::LaunchK*>(a.data());
-    // tensor maps want 64-byte alignment
-    const uintptr_t ta = (reinterpret_cast<uintptr_t>(t.data()) + 63) & ~uintptr_t{63};
-    p.tcargs = reinterpret_cast<ffb::TcLaunchK*>(ta);
-    p.red = reinterpret_cast<ffb::ReduceK*>(r.data());
+    p.args = a.get();
+    p.tcargs = t.get();
+    p.red = r.get();
     return p;
   }
+};
+
+// A launch of structured matrices with its parameters filled.
+struct Ready {
+  Buffers b;
+  Prepared P{};
+  int32_t nm = 0;
 };
 
 // Matrices in the launch that starts at `mats` (`rest` left): the
@@ -635,30 +645,32 @@ size_t structured_workspace(const framefb_mat* mats, int32_t nmats, int32_t ops)
 }
 
 // Validate every launch chunk of the structured matrices; *need = the
-// workspace the largest chunk needs.
+// workspace the largest chunk needs, *ready = the prepared launches.
 framefb_status structured_check(const framefb_mat* mats, int32_t nmats, int32_t ops, framefb_dtype dtype,
-                                size_t* need, const SegTable* seg = nullptr) {
+                                size_t* need, std::vector<Ready>* ready, const SegTable* seg = nullptr) {
   *need = 0;
-  Buffers b;
-  for (int32_t j0 = 0, nm = 0; j0 < nmats; j0 += nm) {
-    nm = chunk_len(mats + j0, nmats - j0, dtype);
-    Prepared P = b.prep();
-    const framefb_status s = prepare(mats + j0, nm, ops, dtype, P, seg);
-    if (s != FRAMEFB_OK) return s;
-    *need = std::max(*need, P.ws_bytes);
+  try {
+    for (int32_t j0 = 0; j0 < nmats; j0 += ready->back().nm) {
+      ready->emplace_back();
+      Ready& r = ready->back();
+      r.nm = chunk_len(mats + j0, nmats - j0, dtype);
+      r.P = r.b.prep();
+      const framefb_status s = prepare(mats + j0, r.nm, ops, dtype, r.P, seg);
+      if (s != FRAMEFB_OK) return s;
+      *need = std::max(*need, r.P.ws_bytes);
+    }
+  } catch (const std::bad_alloc&) {
+    return FRAMEFB_ENOMEM;
   }
   return FRAMEFB_OK;
 }
 
-// Queue the structured kernels (after structured_check).
-framefb_status structured_run(const framefb_mat* mats, int32_t nmats, int32_t ops, framefb_dtype dtype, void* ws,
-                              cudaStream_t st, const SegTable* seg = nullptr) {
-  Buffers b;
-  for (int32_t j0 = 0, nm = 0; j0 < nmats; j0 += nm) {
-    nm = chunk_len(mats + j0, nmats - j0, dtype);
-    Prepared P = b.prep();
-    const framefb_status s = prepare(mats + j0, nm, ops, dtype, P, seg);
-    if (s != FRAMEFB_OK) return s;
+// Queue the launches of structured_check.
+framefb_status structured_run(const std::vector<Ready>& ready, int32_t ops, framefb_dtype dtype, void* ws,
+                              cudaStream_t st) {
+  for (const Ready& r : ready) {
+    const Prepared& P = r.P;
+    const int32_t nm = r.nm;
     if (P.grid == 0) {
       if (ops & FRAMEFB_OP_GRAD_COEFF) {  // no tokens: the gradient is zero
         for (int32_t j = 0; j < nm; ++j)
@@ -862,32 +874,33 @@ extern "C" framefb_status framefb_run(const framefb_mat* mats, int32_t nmats, in
   // validate everything before queueing anything; the waves and the two
   // paths run one after the other on the stream and share the workspace
   size_t need = 0;
+  std::vector<Ready> ready;
   for (const std::vector<framefb_mat>& w : waves) {
     size_t gneed = 0;
-    s = structured_check(w.data(), static_cast<int32_t>(w.size()), ops, dtype, &gneed);
+    s = structured_check(w.data(), static_cast<int32_t>(w.size()), ops, dtype, &gneed, &ready);
     if (s != FRAMEFB_OK) return s;
     need = std::max(need, gneed);
   }
+  ffb_host::RowReady rready;
+  ffb_host::GrpReady fready;
   size_t dneed = 0, rneed = 0;
   s = ffb_host::dense_check(den.data(), static_cast<int32_t>(den.size()), ops, dtype, &dneed);
   if (s != FRAMEFB_OK) return s;
-  s = ffb_host::row_check(row.data(), static_cast<int32_t>(row.size()), ops, dtype, &rneed);
+  s = ffb_host::row_check(row.data(), static_cast<int32_t>(row.size()), ops, dtype, &rneed, &rready);
   if (s != FRAMEFB_OK) return s;
   size_t fneed = 0;
-  s = ffb_host::grp_check(fft.data(), static_cast<int32_t>(fft.size()), ops, dtype, &fneed);
+  s = ffb_host::grp_check(fft.data(), static_cast<int32_t>(fft.size()), ops, dtype, &fneed, &fready);
   if (s != FRAMEFB_OK) return s;
   need = std::max({need, dneed, rneed, fneed});
   if (need > 0) {
     if (!ws || ws_bytes < need) return FRAMEFB_EWORKSPACE;
     if (reinterpret_cast<uintptr_t>(ws) & 255u) return FRAMEFB_EINVAL;
   }
-  for (const std::vector<framefb_mat>& w : waves) {
-    s = structured_run(w.data(), static_cast<int32_t>(w.size()), ops, dtype, ws, st);
-    if (s != FRAMEFB_OK) return s;
-  }
-  s = ffb_host::grp_run(fft.data(), static_cast<int32_t>(fft.size()), ops, dtype, ws, st);
+  s = structured_run(ready, ops, dtype, ws, st);
   if (s != FRAMEFB_OK) return s;
-  s = ffb_host::row_run(row.data(), static_cast<int32_t>(row.size()), ops, dtype, ws, st);
+  s = ffb_host::grp_run(fready, ws, st);
+  if (s != FRAMEFB_OK) return s;
+  s = ffb_host::row_run(rready, ws, st);
   if (s != FRAMEFB_OK) return s;
   return ffb_host::dense_run(den.data(), static_cast<int32_t>(den.size()), ops, dtype, ws, ws_bytes, st);
 }
@@ -1040,10 +1053,10 @@ extern "C" framefb_status framefb_forward_tenants(const framefb_mat* mats, int32
     if (den.empty() && row.empty() && fft.empty()) {
       const SegTable st{nseg, seg_start, seg_tenant};
       size_t need = 0;
-      s = structured_check(grp.data(), static_cast<int32_t>(grp.size()), FRAMEFB_OP_FORWARD, dtype, &need, &st);
+      std::vector<Ready> ready;
+      s = structured_check(grp.data(), static_cast<int32_t>(grp.size()), FRAMEFB_OP_FORWARD, dtype, &need, &ready, &st);
       if (s == FRAMEFB_OK)
-        return structured_run(grp.data(), static_cast<int32_t>(grp.size()), FRAMEFB_OP_FORWARD, dtype, nullptr,
-                              static_cast<cudaStream_t>(stream), &st);
+        return structured_run(ready, FRAMEFB_OP_FORWARD, dtype, nullptr, static_cast<cudaStream_t>(stream));
       if (s != FRAMEFB_EUNSUPPORTED) return s;
     }
   }

@@ -5,6 +5,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <cstddef>
 #include <cstring>
 #include <memory>
 #include <new>
@@ -180,8 +181,9 @@ std::vector<Chunk> chunks_of(const framefb_mat* mats, int32_t nmats) {
 }
 
 framefb_status prepare(const Chunk& ch, int32_t ops, framefb_dtype dt, Prepared& P) {
-  std::memset(P.args, 0, sizeof(fg::Launch));
-  std::memset(P.red, 0, sizeof(fp::Reduce));
+  // (the matrices' entries are filled below, the rest is never read)
+  std::memset(P.args, 0, offsetof(fg::Launch, m));
+  std::memset(P.red, 0, offsetof(fp::Reduce, m));
   fg::Launch& A = *P.args;
   P.v = ch.v;
   void* fn = kernel_ptr(ch.v, dt);
@@ -348,7 +350,19 @@ bool grp_takes(const framefb_mat& M, int32_t ops, framefb_dtype dt) {
   return v.big && (h->Gm > 128 || (h->Gn > 128 && M.N >= kMinTokensWideIn));
 }
 
-framefb_status grp_check(const framefb_mat* mats, int32_t nmats, int32_t ops, framefb_dtype dt, size_t* ws_need) {
+struct GrpLaunches {
+  struct One {
+    Buffers b;
+    Prepared P{};
+    void* fn = nullptr;
+    unsigned mats = 0;
+    bool reduce = false;
+  };
+  std::vector<One> list;
+};
+
+framefb_status grp_check(const framefb_mat* mats, int32_t nmats, int32_t ops, framefb_dtype dt, size_t* ws_need,
+                         GrpReady* keep) {
   *ws_need = 0;
   if (nmats == 0) return FRAMEFB_OK;
   for (int32_t j = 0; j < nmats; ++j) {
@@ -356,42 +370,39 @@ framefb_status grp_check(const framefb_mat* mats, int32_t nmats, int32_t ops, fr
     if (s != FRAMEFB_OK) return s;
   }
   try {
-    Buffers b;
+    auto all = std::make_shared<GrpLaunches>();
     for (const Chunk& c : chunks_of(mats, nmats)) {
-      Prepared P = b.prep();
-      const framefb_status s = prepare(c, ops, dt, P);
+      if (keep || all->list.empty()) all->list.emplace_back();
+      GrpLaunches::One& l = all->list.back();
+      l.P = l.b.prep();
+      const framefb_status s = prepare(c, ops, dt, l.P);
       if (s != FRAMEFB_OK) return s;
-      *ws_need = std::max(*ws_need, P.ws_bytes);
+      *ws_need = std::max(*ws_need, l.P.ws_bytes);
+      l.fn = kernel_ptr(l.P.v, dt);
+      l.mats = static_cast<unsigned>(c.mats.size());
+      l.reduce = (ops & FRAMEFB_OP_GRAD_COEFF) && l.P.nnz_max > 0;
     }
+    if (keep) *keep = std::move(all);
   } catch (const std::bad_alloc&) {
     return FRAMEFB_ENOMEM;
   }
   return FRAMEFB_OK;
 }
 
-framefb_status grp_run(const framefb_mat* mats, int32_t nmats, int32_t ops, framefb_dtype dt, void* ws, cudaStream_t st) {
-  if (nmats == 0) return FRAMEFB_OK;
-  try {
-    Buffers b;
-    for (const Chunk& c : chunks_of(mats, nmats)) {
-      Prepared P = b.prep();
-      const framefb_status s = prepare(c, ops, dt, P);
-      if (s != FRAMEFB_OK) return s;
-      P.args->partial = static_cast<float*>(ws);
-      P.red->partial = static_cast<const float*>(ws);
-      void* kargs[] = {P.args};
-      if (launch_chained(kernel_ptr(P.v, dt), dim3(P.grid), dim3(P.v.nt), kargs, P.smem, st) != cudaSuccess)
+framefb_status grp_run(const GrpReady& ready, void* ws, cudaStream_t st) {
+  if (!ready) return FRAMEFB_OK;
+  for (const GrpLaunches::One& l : ready->list) {
+    const Prepared& P = l.P;
+    P.args->partial = static_cast<float*>(ws);
+    P.red->partial = static_cast<const float*>(ws);
+    void* kargs[] = {P.args};
+    if (launch_chained(l.fn, dim3(P.grid), dim3(P.v.nt), kargs, P.smem, st) != cudaSuccess) return FRAMEFB_ECUDA;
+    if (l.reduce) {
+      void* rargs[] = {P.red};
+      if (launch_chained(reinterpret_cast<void*>(fp::pair_reduce_kernel), dim3((P.nnz_max + 31) / 32, l.mats),
+                         dim3(32 * fp::kLanes), rargs, 0, st) != cudaSuccess)
         return FRAMEFB_ECUDA;
-      if ((ops & FRAMEFB_OP_GRAD_COEFF) && P.nnz_max > 0) {
-        void* rargs[] = {P.red};
-        if (launch_chained(reinterpret_cast<void*>(fp::pair_reduce_kernel),
-                             dim3((P.nnz_max + 31) / 32, static_cast<unsigned>(c.mats.size())), dim3(32 * fp::kLanes), rargs,
-                             0, st) != cudaSuccess)
-          return FRAMEFB_ECUDA;
-      }
     }
-  } catch (const std::bad_alloc&) {
-    return FRAMEFB_ENOMEM;
   }
   return FRAMEFB_OK;
 }

@@ -3,6 +3,8 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <memory>
+
 #include "framefb.h"
 
 namespace ffb_host {
@@ -10,12 +12,17 @@ namespace ffb_host {
 // Whether a matrix of a call runs on the group-transform kernel.
 bool grp_takes(const framefb_mat& M, int32_t ops, framefb_dtype dt);
 
-// Validate the path's matrices and report the workspace they need (bytes;
-// the launches run one after another and share it).
-framefb_status grp_check(const framefb_mat* mats, int32_t nmats, int32_t ops, framefb_dtype dt, size_t* ws_need);
+// The launches of a call, with their parameters filled.
+struct GrpLaunches;
+using GrpReady = std::shared_ptr<GrpLaunches>;
 
-// Queue the path on `st` (after grp_check).
-framefb_status grp_run(const framefb_mat* mats, int32_t nmats, int32_t ops, framefb_dtype dt, void* ws,
-                       cudaStream_t st);
+// Validate the path's matrices, report the workspace they need (bytes; the
+// launches run one after another and share it), and hand the prepared
+// launches on through `keep`.
+framefb_status grp_check(const framefb_mat* mats, int32_t nmats, int32_t ops, framefb_dtype dt, size_t* ws_need,
+                         GrpReady* keep = nullptr);
+
+// Queue the launches of grp_check on `st` (none if `ready` is empty).
+framefb_status grp_run(const GrpReady& ready, void* ws, cudaStream_t st);
 
 }  // namespace ffb_host

@@ -5,6 +5,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <cstddef>
 #include <cstdlib>
 #include <cstring>
 #include <memory>
@@ -188,8 +189,9 @@ std::vector<Chunk> chunks_of(const framefb_mat* mats, int32_t nmats) {
 }
 
 framefb_status prepare(const Chunk& ch, int32_t ops, Prepared& P) {
-  std::memset(P.args, 0, sizeof(fr::Launch));
-  std::memset(P.red, 0, sizeof(fp::Reduce));
+  // (the matrices' entries are filled below, the rest is never read)
+  std::memset(P.args, 0, offsetof(fr::Launch, m));
+  std::memset(P.red, 0, offsetof(fp::Reduce, m));
   fr::Launch& A = *P.args;
   P.v = ch.v;
   void* fn = kernel_ptr(ch.v);
@@ -325,49 +327,57 @@ bool row_takes(const framefb_mat& M, int32_t ops, framefb_dtype dt) {
   return variant(M, sh).nt != 0;
 }
 
-framefb_status row_check(const framefb_mat* mats, int32_t nmats, int32_t ops, framefb_dtype, size_t* ws_need) {
+struct RowLaunches {
+  struct One {
+    Buffers b;
+    Prepared P{};
+    void* fn = nullptr;
+    unsigned mats = 0;
+    bool reduce = false;
+  };
+  std::vector<One> list;
+};
+
+framefb_status row_check(const framefb_mat* mats, int32_t nmats, int32_t ops, framefb_dtype, size_t* ws_need,
+                         RowReady* keep) {
   *ws_need = 0;
   if (nmats == 0) return FRAMEFB_OK;
   for (int32_t j = 0; j < nmats; ++j)
     if (!dense_mat_ok(mats[j], ops)) return FRAMEFB_EINVAL;
   try {
-    Buffers b;
+    auto all = std::make_shared<RowLaunches>();
     for (const Chunk& c : chunks_of(mats, nmats)) {
-      Prepared P = b.prep();
-      const framefb_status s = prepare(c, ops, P);
+      if (keep || all->list.empty()) all->list.emplace_back();
+      RowLaunches::One& l = all->list.back();
+      l.P = l.b.prep();
+      const framefb_status s = prepare(c, ops, l.P);
       if (s != FRAMEFB_OK) return s;
-      *ws_need = std::max(*ws_need, P.ws_bytes);
+      *ws_need = std::max(*ws_need, l.P.ws_bytes);
+      l.fn = kernel_ptr(l.P.v);
+      l.mats = static_cast<unsigned>(c.mats.size());
+      l.reduce = (ops & FRAMEFB_OP_GRAD_COEFF) && l.P.nnz_max > 0;
     }
+    if (keep) *keep = std::move(all);
   } catch (const std::bad_alloc&) {
     return FRAMEFB_ENOMEM;
   }
   return FRAMEFB_OK;
 }
 
-framefb_status row_run(const framefb_mat* mats, int32_t nmats, int32_t ops, framefb_dtype, void* ws,
-                       cudaStream_t st) {
-  if (nmats == 0) return FRAMEFB_OK;
-  try {
-    Buffers b;
-    for (const Chunk& c : chunks_of(mats, nmats)) {
-      Prepared P = b.prep();
-      const framefb_status s = prepare(c, ops, P);
-      if (s != FRAMEFB_OK) return s;
-      P.args->partial = static_cast<float*>(ws);
-      P.red->partial = static_cast<const float*>(ws);
-      void* kargs[] = {P.args};
-      if (launch_chained(kernel_ptr(P.v), dim3(P.grid), dim3(P.v.nt), kargs, P.smem, st) != cudaSuccess)
+framefb_status row_run(const RowReady& ready, void* ws, cudaStream_t st) {
+  if (!ready) return FRAMEFB_OK;
+  for (const RowLaunches::One& l : ready->list) {
+    const Prepared& P = l.P;
+    P.args->partial = static_cast<float*>(ws);
+    P.red->partial = static_cast<const float*>(ws);
+    void* kargs[] = {P.args};
+    if (launch_chained(l.fn, dim3(P.grid), dim3(P.v.nt), kargs, P.smem, st) != cudaSuccess) return FRAMEFB_ECUDA;
+    if (l.reduce) {
+      void* rargs[] = {P.red};
+      if (launch_chained(reinterpret_cast<void*>(fp::pair_reduce_kernel), dim3((P.nnz_max + 31) / 32, l.mats),
+                         dim3(32 * fp::kLanes), rargs, 0, st) != cudaSuccess)
         return FRAMEFB_ECUDA;
-      if ((ops & FRAMEFB_OP_GRAD_COEFF) && P.nnz_max > 0) {
-        void* rargs[] = {P.red};
-        if (launch_chained(reinterpret_cast<void*>(fp::pair_reduce_kernel),
-                             dim3((P.nnz_max + 31) / 32, static_cast<unsigned>(c.mats.size())), dim3(32 * fp::kLanes), rargs,
-                             0, st) != cudaSuccess)
-          return FRAMEFB_ECUDA;
-      }
     }
-  } catch (const std::bad_alloc&) {
-    return FRAMEFB_ENOMEM;
   }
   return FRAMEFB_OK;
 }
