@@ -31,7 +31,7 @@ NOMINAL_GBS = 8000.0
 L2_BYTES = 126 * 1024 * 1024
 
 # evaluation workloads reported in per_config, in the order of their configs,
-# then the paper's own rho = 2 regime at the LLaMA-2 shape (the dense path)
+# then the paper's own rho = 2 regime at the LLaMA-2 shape
 PER_CONFIG = ("single_256_fp32", "roberta_base_qv", "llama2_7b_qkvo", "llama3_8b_all", "vit_b16_merge",
               "llama2_rho2")
 
@@ -379,9 +379,9 @@ def time_config(name, dev, stream, steps, warmup, flush, with_cpu, headline=None
         batch = AdapterBatch(w, dev, ops=ops)
         ws = batch.workspace(ops)
         alg = algorithmic_bytes(batch)
-        if not all(f.structured for f in batch.frames.values()):
-            flops = dense_flops(batch)
         kernels = ffb.framefb_kernel_names(batch.mats, ops, batch.dtype_code)
+        if any(k.startswith("dense") for k in kernels) and not all(f.structured for f in batch.frames.values()):
+            flops = dense_flops(batch)
         small = alg < 2 * L2_BYTES
         ms = time_steps(lambda: batch.run(ops, ws, stream), stream, steps, warmup, flush if small else None)
         del batch, ws
@@ -390,7 +390,8 @@ def time_config(name, dev, stream, steps, warmup, flush, with_cpu, headline=None
     rec = {"ms_per_step": ms, "tokens_per_s": w.N / (ms / 1e3), "matrices": len(w.mats), "tokens": w.N,
            "dtype": w.dtype, "algorithmic_bytes": alg, "achieved_gbs": gbs, "frac_of_measured": gbs / peak,
            "frac_of_8tbs": gbs / NOMINAL_GBS,
-           "kernels": kernels + ([] if any(k.startswith("dense") for k in kernels) else ["dc_reduce_kernel"]),
+           "kernels": kernels + (["dc_reduce_kernel"] if any(k.startswith(("tc", "mma")) for k in kernels) else [])
+           + (["pair_reduce_kernel"] if any(k.startswith(("row", "fft")) for k in kernels) else []),
            "l2": "L2 flushed between steps" if alg < 2 * L2_BYTES else "step moves more than L2"}
     if flops:
         tpk, kind = tensor_peak()
