@@ -550,9 +550,7 @@ framefb_status prepare(const framefb_mat* mats, int32_t nmats, int32_t ops, fram
   int dev = 0, sms = 0, per_sm = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return FRAMEFB_ECUDA;
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return FRAMEFB_ECUDA;
-  if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(P.smem)) !=
-      cudaSuccess)
-    return FRAMEFB_ECUDA;
+  if (ffb_host::allow_shared(fn, dev, P.smem) != cudaSuccess) return FRAMEFB_ECUDA;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, P.threads, P.smem) != cudaSuccess)
     return FRAMEFB_ECUDA;
   if (per_sm < 1) return FRAMEFB_EUNSUPPORTED;

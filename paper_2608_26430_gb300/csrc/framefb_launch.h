@@ -14,6 +14,21 @@
 
 namespace ffb_host {
 
+// Lets `fn` take `smem` bytes of dynamic shared memory.  The limit is always set
+// to all that a CTA of the kernel can have: a call prepares its launches before
+// it queues the first, and other threads prepare theirs, so no launch may depend
+// on the size that was set last.
+inline cudaError_t allow_shared(const void* fn, int dev, size_t smem) {
+  cudaFuncAttributes fa{};
+  int optin = 0;
+  cudaError_t e = cudaFuncGetAttributes(&fa, fn);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e != cudaSuccess) return e;
+  const size_t most = static_cast<size_t>(optin) - fa.sharedSizeBytes;
+  if (smem > most) return cudaErrorInvalidValue;
+  return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(most));
+}
+
 inline cudaError_t launch_chained(void* fn, dim3 grid, dim3 block, void** args, size_t smem, cudaStream_t st) {
   cudaLaunchAttribute at{};
   at.id = cudaLaunchAttributeProgrammaticStreamSerialization;

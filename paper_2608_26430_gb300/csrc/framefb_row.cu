@@ -272,7 +272,7 @@ framefb_status prepare(const Chunk& ch, int32_t ops, Prepared& P) {
   A.stride = (nnz_max + 63) & ~63;
   P.nnz_max = nnz_max;
   int per_sm = 0;
-  if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(P.smem)) != cudaSuccess ||
+  if (allow_shared(fn, dev, P.smem) != cudaSuccess ||
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, ch.v.nt, P.smem) != cudaSuccess)
     return FRAMEFB_ECUDA;
   if (per_sm < 1) return FRAMEFB_EUNSUPPORTED;

@@ -30,7 +30,9 @@ def built():
 # kernels, with grids of a few CTAs and of every SM
 SHAPES = [("f32", [(256, 256)], 8, 128, False), ("f32", [(768, 768)] * 4, 700, 1000, False),
           ("bf16", [(256, 256)], 33, 200, False), ("bf16", [(768, 768)] * 6, 1500, 1000, False),
-          ("bf16", [(4096, 4096)], 37, 4096, False), ("bf16", [(1024, 1024)] * 2, 301, 900, True)]
+          ("bf16", [(4096, 4096)], 37, 4096, False), ("bf16", [(1024, 1024)] * 2, 301, 900, True),
+          # one kernel in two launches, the second with less shared memory
+          ("bf16", [(768, 768), (1024, 256)], 77, 600, False)]
 
 
 def build_batch(shape):
