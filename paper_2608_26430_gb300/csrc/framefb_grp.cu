@@ -13,6 +13,7 @@
 #include <vector>
 
 #include "framefb.h"
+#include "framefb_dense.h"
 #include "framefb_grp.cuh"
 #include "framefb_grp.h"
 #include "framefb_launch.h"
@@ -366,8 +367,16 @@ framefb_status grp_check(const framefb_mat* mats, int32_t nmats, int32_t ops, fr
   *ws_need = 0;
   if (nmats == 0) return FRAMEFB_OK;
   for (int32_t j = 0; j < nmats; ++j) {
-    const framefb_status s = check_mat(mats[j], ops, dt);
+    framefb_status s = check_mat(mats[j], ops, dt);
     if (s != FRAMEFB_OK) return s;
+    // the workspace asked for covers fewer tokens too, where the contraction
+    // path takes these plans (kMinTokensWideIn)
+    if (dt == FRAMEFB_BF16 && header_of(mats[j].plan)->Gn > 128 && mats[j].ldx == mats[j].n && mats[j].ldy == mats[j].m) {
+      size_t need = 0;
+      s = dense_check(&mats[j], 1, ops, dt, &need);
+      if (s != FRAMEFB_OK) return s;
+      *ws_need = std::max(*ws_need, need);
+    }
   }
   try {
     auto all = std::make_shared<GrpLaunches>();

@@ -338,12 +338,17 @@ struct RowLaunches {
   std::vector<One> list;
 };
 
-framefb_status row_check(const framefb_mat* mats, int32_t nmats, int32_t ops, framefb_dtype, size_t* ws_need,
+// The workspace asked for stays the contraction path's, though this path needs
+// only its dC partials: which of the two a call takes depends on its tokens, and
+// callers size one workspace for calls that differ in them.
+framefb_status row_check(const framefb_mat* mats, int32_t nmats, int32_t ops, framefb_dtype dt, size_t* ws_need,
                          RowReady* keep) {
   *ws_need = 0;
   if (nmats == 0) return FRAMEFB_OK;
   for (int32_t j = 0; j < nmats; ++j)
     if (!dense_mat_ok(mats[j], ops)) return FRAMEFB_EINVAL;
+  const framefb_status d = dense_check(mats, nmats, ops, dt, ws_need);
+  if (d != FRAMEFB_OK) return d;
   try {
     auto all = std::make_shared<RowLaunches>();
     for (const Chunk& c : chunks_of(mats, nmats)) {

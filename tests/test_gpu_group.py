@@ -89,6 +89,13 @@ def test_bf16_wide_sides(mats, N):
     check(AdapterBatch(load(mats, N, 4300, "bf16", support_mode=wl.ZIPF_ROWS), DEV, ops=ALL), ALL)
 
 
+def test_workspace_covers_fewer_tokens():
+    """One workspace serves calls of fewer tokens, whichever path takes them."""
+    sizes = [ffb.framefb_workspace_size(AdapterBatch(load([(4608, 256)], N, 4300, "bf16", support_mode=wl.ZIPF_ROWS), DEV,
+                                                     ops=ALL).mats, ALL) for N in (3, 127, 128, 400)]
+    assert sizes == sorted(sizes)
+
+
 def test_entry_points_agree():
     w = load([(768, 768), (1024, 768)], 50, 1500)
     a, s = AdapterBatch(w, DEV, ops=ALL), AdapterBatch(w, DEV, ops=ALL)

@@ -133,6 +133,13 @@ def test_padded_rows_and_empty_support():
     assert torch.equal(e.bufs[0].Y, Y0) and torch.equal(e.bufs[0].dX, X0)
 
 
+def test_workspace_covers_fewer_tokens():
+    """One workspace serves calls of fewer tokens, whichever path takes them."""
+    sizes = [ffb.framefb_workspace_size(AdapterBatch(rho2([(768, 768)], N, 1000), DEV, ops=ALL).mats, ALL)
+             for N in (1, 511, 512, 900)]
+    assert sizes == sorted(sizes)
+
+
 def test_more_matrices_than_a_launch_holds():
     w = rho2([(256, 256)] * 100, 5, 100)
     b = AdapterBatch(w, DEV, ops=ALL)
