@@ -276,17 +276,17 @@ __device__ __forceinline__ void load_cols(Cols& ch, uint8_t* sp, int mode, const
     float zc = 0.f, gc = 0.f;
     const int ez = half * ch.hZ + i, eg = half * ch.hG + i;
     if (i < ch.hZ && ez < h.EZ) {
-      zw = word(static_cast<uint32_t>(__ldg(tab(h.off_zb) + ez * kColumns + col)), 1);
-      const int32_t qi = __ldg(tab(h.off_zq) + ez * kColumns + col);
-      zc = qi >= 0 ? __ldg(c_val + qi) : 0.f;
+      zw = word(static_cast<uint32_t>(ld_g(tab(h.off_zb) + ez * kColumns + col)), 1);
+      const int32_t qi = ld_g(tab(h.off_zq) + ez * kColumns + col);
+      zc = qi >= 0 ? ld_g(c_val + qi) : 0.f;
       openZ = qi >= 0 && (zw >> 16) == FFB_NO_STORE;
       if (firstZ == FFB_NO_STORE) firstZ = zw >> 16;
     }
     if (i < ch.hG && eg < h.EG) {
-      gw = word(static_cast<uint32_t>(__ldg(tab(h.off_ga) + eg * kColumns + col)), 0);
-      gb = 8u * col_slot(static_cast<uint32_t>(__ldg(tab(h.off_gb) + eg * kColumns + col)));
-      const int32_t qi = __ldg(tab(h.off_gq) + eg * kColumns + col);
-      gc = (D && qi >= 0) ? __ldg(c_val + qi) : 0.f;
+      gw = word(static_cast<uint32_t>(ld_g(tab(h.off_ga) + eg * kColumns + col)), 0);
+      gb = 8u * col_slot(static_cast<uint32_t>(ld_g(tab(h.off_gb) + eg * kColumns + col)));
+      const int32_t qi = ld_g(tab(h.off_gq) + eg * kColumns + col);
+      gc = (D && qi >= 0) ? ld_g(c_val + qi) : 0.f;
       openG = qi >= 0 && (gw >> 16) == FFB_NO_STORE;
       if (firstG == FFB_NO_STORE) firstG = gw >> 16;
       if (!D) gw |= FFB_NO_STORE << 16;
@@ -418,23 +418,23 @@ __device__ __forceinline__ void load_big(Big& ch, uint8_t* sp, int mode, const u
     float zc = 0.f, gc = 0.f;
     const int ez = half * ch.hZ + i, eg = half * ch.hG + i;
     if (i < ch.hZ && ez < h.EZ) {
-      const uint32_t w = static_cast<uint32_t>(__ldg(tab(h.off_zb) + ez * kColumns + col));
-      const int32_t qi = __ldg(tab(h.off_zq) + ez * kColumns + col);
+      const uint32_t w = static_cast<uint32_t>(ld_g(tab(h.off_zb) + ez * kColumns + col));
+      const int32_t qi = ld_g(tab(h.off_zq) + ez * kColumns + col);
       const uint32_t t = (w >> 16) == FFB_NO_STORE ? kNoZ : target(w >> 16, 1);
       // (padding entries carry column 0: slot 0 of the buffer, with value 0)
       z = (qi >= 0 ? slot(0, w & 0x7FFFu) : 0u) | (t << 13);
-      zc = qi >= 0 ? __ldg(c_val + qi) : 0.f;
+      zc = qi >= 0 ? ld_g(c_val + qi) : 0.f;
       openZ = qi >= 0 && t == kNoZ;
       if (firstZ == kNoZ) firstZ = t;
     }
     if (i < ch.hG && eg < h.EG) {
-      const uint32_t w = static_cast<uint32_t>(__ldg(tab(h.off_ga) + eg * kColumns + col));
-      const int32_t qi = __ldg(tab(h.off_gq) + eg * kColumns + col);
+      const uint32_t w = static_cast<uint32_t>(ld_g(tab(h.off_ga) + eg * kColumns + col));
+      const int32_t qi = ld_g(tab(h.off_gq) + eg * kColumns + col);
       const uint32_t t = (w >> 16) == FFB_NO_STORE || !D ? kNoG : target(w >> 16, 0);
-      const uint32_t b = qi >= 0 ? slot(0, static_cast<uint32_t>(__ldg(tab(h.off_gb) + eg * kColumns + col))) : 0u;
+      const uint32_t b = qi >= 0 ? slot(0, static_cast<uint32_t>(ld_g(tab(h.off_gb) + eg * kColumns + col))) : 0u;
       g = (qi >= 0 ? slot(1, w & 0x7FFFu) : 0u) | (t << 12) | ((b >> 7) << 25);
       z |= (b & 127u) << 25;
-      gc = (D && qi >= 0) ? __ldg(c_val + qi) : 0.f;
+      gc = (D && qi >= 0) ? ld_g(c_val + qi) : 0.f;
       openG = D && qi >= 0 && t == kNoG;
       if (firstG == kNoG) firstG = t;
     }
@@ -634,7 +634,7 @@ __global__ void __launch_bounds__(NT, NT == 512 ? 1 : 2) group_kernel(const __gr
       for (int i = 0; i < ch.hG; ++i) {
         const int e = half * ch.hG + i;
         if (e < h.EG) {
-          const int32_t qi = __ldg(gq + e * kColumns + col);
+          const int32_t qi = ld_g(gq + e * kColumns + col);
           if (qi >= 0) dst[qi] = arr[((2 * (kBigE / 4) + i / 4) * NT + tid) * 4 + (i & 3)];
         }
       }
@@ -680,7 +680,7 @@ __global__ void __launch_bounds__(NT, NT == 512 ? 1 : 2) group_kernel(const __gr
       }
       const uint32_t* gm = reinterpret_cast<const uint32_t*>(plan + h.off_gmask);
       const uint32_t* zm = reinterpret_cast<const uint32_t*>(plan + h.off_zmask);
-      for (int g = tid; g < G0 + G1; g += NT) masks[g] = g < G0 ? __ldg(gm + g) : __ldg(zm + (g - G0));
+      for (int g = tid; g < G0 + G1; g += NT) masks[g] = g < G0 ? ld_g(gm + g) : ld_g(zm + (g - G0));
       // run-sum slots that no run writes read as zero
       for (int x = tid; x < PP * sh.pair; x += NT) pairs[x] = make_float2(0.f, 0.f);
       __syncthreads();

@@ -105,16 +105,16 @@ struct Tw {
 
 __device__ __forceinline__ Tw load_tw(const float* v) {
   Tw w;
-  w.c1 = 4.f * __ldg(v + 2);
-  w.s1 = -4.f * __ldg(v + 3);
-  w.c2 = 4.f * __ldg(v + 4);
-  w.s2 = -4.f * __ldg(v + 5);
-  w.c3 = 4.f * __ldg(v + 6);
-  w.s3 = -4.f * __ldg(v + 7);
-  w.c6 = 4.f * __ldg(v + 12);
-  w.s6 = -4.f * __ldg(v + 13);
-  w.c9 = 4.f * __ldg(v + 18);
-  w.s9 = -4.f * __ldg(v + 19);
+  w.c1 = 4.f * ld_g(v + 2);
+  w.s1 = -4.f * ld_g(v + 3);
+  w.c2 = 4.f * ld_g(v + 4);
+  w.s2 = -4.f * ld_g(v + 5);
+  w.c3 = 4.f * ld_g(v + 6);
+  w.s3 = -4.f * ld_g(v + 7);
+  w.c6 = 4.f * ld_g(v + 12);
+  w.s6 = -4.f * ld_g(v + 13);
+  w.c9 = 4.f * ld_g(v + 18);
+  w.s9 = -4.f * ld_g(v + 19);
   return w;
 }
 
@@ -364,17 +364,17 @@ struct Chunk {
 #pragma unroll
       for (int e = 0; e < E; ++e) {
         if (F && e < EZ) {
-          const uint32_t w = static_cast<uint32_t>(__ldg(tzb + e * kThreads + tid));
+          const uint32_t w = static_cast<uint32_t>(ld_g(tzb + e * kThreads + tid));
           zb[e] = slots(w, n, m);
-          const int32_t q = __ldg(tzq + e * kThreads + tid);
-          zc[e] = q >= 0 ? signed_c(__ldg(c_val + q), w) : 0.f;
+          const int32_t q = ld_g(tzq + e * kThreads + tid);
+          zc[e] = q >= 0 ? signed_c(ld_g(c_val + q), w) : 0.f;
         }
         if ((D || C) && e < EG) {
-          const uint32_t w = static_cast<uint32_t>(__ldg(tga + e * kThreads + tid));
+          const uint32_t w = static_cast<uint32_t>(ld_g(tga + e * kThreads + tid));
           ga[e] = slots(w, m, n);
-          gb[e] = static_cast<uint32_t>(ffb_slot(__ldg(tgb + e * kThreads + tid), n));
-          const int32_t q = __ldg(tgq + e * kThreads + tid);
-          gc[e] = (D && q >= 0) ? signed_c(__ldg(c_val + q), w) : 0.f;
+          gb[e] = static_cast<uint32_t>(ffb_slot(ld_g(tgb + e * kThreads + tid), n));
+          const int32_t q = ld_g(tgq + e * kThreads + tid);
+          gc[e] = (D && q >= 0) ? signed_c(ld_g(c_val + q), w) : 0.f;
         }
       }
     }
@@ -391,10 +391,10 @@ struct Chunk {
       w = zb[e];
       c = zc[e];
     } else {
-      const uint32_t raw = static_cast<uint32_t>(__ldg(table<int32_t>(plan, hdr(plan).off_zb) + e * kThreads + tid));
+      const uint32_t raw = static_cast<uint32_t>(ld_g(table<int32_t>(plan, hdr(plan).off_zb) + e * kThreads + tid));
       w = slots(raw, n, m);
-      const int32_t q = __ldg(table<int32_t>(plan, hdr(plan).off_zq) + e * kThreads + tid);
-      c = q >= 0 ? signed_c(__ldg(c_val + q), raw) : 0.f;
+      const int32_t q = ld_g(table<int32_t>(plan, hdr(plan).off_zq) + e * kThreads + tid);
+      c = q >= 0 ? signed_c(ld_g(c_val + q), raw) : 0.f;
     }
   }
   __device__ __forceinline__ void g_entry(const uint8_t* plan, const float* c_val, int tid, int e, uint32_t& wa,
@@ -407,13 +407,13 @@ struct Chunk {
       wb = gb[e];
       c = gc[e];
     } else {
-      const uint32_t raw = static_cast<uint32_t>(__ldg(table<int32_t>(plan, hdr(plan).off_ga) + e * kThreads + tid));
+      const uint32_t raw = static_cast<uint32_t>(ld_g(table<int32_t>(plan, hdr(plan).off_ga) + e * kThreads + tid));
       wa = slots(raw, m, n);
-      wb = static_cast<uint32_t>(ffb_slot(__ldg(table<int32_t>(plan, hdr(plan).off_gb) + e * kThreads + tid), n));
+      wb = static_cast<uint32_t>(ffb_slot(ld_g(table<int32_t>(plan, hdr(plan).off_gb) + e * kThreads + tid), n));
       c = 0.f;
       if constexpr (D) {
-        const int32_t q = __ldg(table<int32_t>(plan, hdr(plan).off_gq) + e * kThreads + tid);
-        c = q >= 0 ? signed_c(__ldg(c_val + q), raw) : 0.f;
+        const int32_t q = ld_g(table<int32_t>(plan, hdr(plan).off_gq) + e * kThreads + tid);
+        c = q >= 0 ? signed_c(ld_g(c_val + q), raw) : 0.f;
       }
     }
   }
@@ -560,7 +560,7 @@ struct Chunk {
       const int32_t* gq = table<int32_t>(plan, hdr(plan).off_gq);
       const float* dcs = fsm + L.oDC;
       for (int e = 0; e < EG; ++e) {
-        const int32_t q = __ldg(gq + e * kThreads + tid);
+        const int32_t q = ld_g(gq + e * kThreads + tid);
         if (q >= 0) dst[q] = dcs[e * kThreads + tid];
       }
     }
@@ -579,7 +579,7 @@ __device__ __forceinline__ void fixup(const uint8_t* plan, const FfbTileLayout& 
   const int nfZ = F ? h.nfixZ : 0, nfG = D ? h.nfixG : 0;
   for (int i = tid; i < nfZ + nfG; i += NT) {
     const bool z = i < nfZ;
-    const int4 it = z ? __ldg(table<int4>(plan, h.off_fixZ) + i) : __ldg(table<int4>(plan, h.off_fixG) + (i - nfZ));
+    const int4 it = z ? ld_g(table<int4>(plan, h.off_fixZ) + i) : ld_g(table<int4>(plan, h.off_fixG) + (i - nfZ));
     float* R = fsm + (z ? L.oRZ : L.oRG);
     const int stride = z ? L.sRZ : L.sRG;
     const int dst = ffb_slot(it.x, z ? h.m : h.n);
@@ -672,7 +672,7 @@ __global__ void __launch_bounds__(kThreads, 1) fft_tile_kernel(const __grid_cons
         const bool isV = NEED_V && g < (NEED_V ? Gn : 0);
         if (!isV && NEED_V) g -= Gn;
         if (isV) {
-          if (__ldg(gmask + g) == 0u) continue;
+          if (ld_g(gmask + g) == 0u) continue;
           Seg<Elem> s;
           s.load_stream(static_cast<const char*>(M.X) + ((t0 + t) * M.ldx + 32 * g) * ELEM);
           float xr[16], xi[16];
@@ -680,7 +680,7 @@ __global__ void __launch_bounds__(kThreads, 1) fft_tile_kernel(const __grid_cons
           fft16<+1>(xr, xi, tw_in);
           store_group(V + t * L.sV, g, xr, xi);
         } else {
-          if (__ldg(zmask + g) == 0u) continue;
+          if (ld_g(zmask + g) == 0u) continue;
           Seg<Elem> s;
           s.load_stream(static_cast<const char*>(M.dY) + ((t0 + t) * M.ldy + 32 * g) * ELEM);
           float xr[16], xi[16];
@@ -710,7 +710,7 @@ __global__ void __launch_bounds__(kThreads, 1) fft_tile_kernel(const __grid_cons
         const bool isY = F && g < (F ? Gm : 0);
         if (!isY && F) g -= Gm;
         if (isY) {
-          if (__ldg(zmask + g) == 0u) continue;
+          if (ld_g(zmask + g) == 0u) continue;
           char* yp = static_cast<char*>(M.Y) + ((t0 + t) * M.ldy + 32 * g) * ELEM;
           Seg<Elem> s;
           s.load(yp);
@@ -719,7 +719,7 @@ __global__ void __launch_bounds__(kThreads, 1) fft_tile_kernel(const __grid_cons
           fft16<-1>(xr, xi, tw_out);
           s.add_store(yp, xr, xi, M.seff);
         } else {
-          if (__ldg(gmask + g) == 0u) continue;
+          if (ld_g(gmask + g) == 0u) continue;
           char* xp = static_cast<char*>(M.dX) + ((t0 + t) * M.ldx + 32 * g) * ELEM;
           Seg<Elem> s;
           s.load(xp);
@@ -746,7 +746,7 @@ __global__ void __launch_bounds__(256) dc_reduce_kernel(const __grid_constant__ 
   const ReduceMat& M = r.m[j];
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= M.nnz) return;
-  const int q = M.qlist ? __ldg(M.qlist + i) : i;
+  const int q = M.qlist ? ld_g(M.qlist + i) : i;
   float s = 0.f;
   if (M.ntiles > 0) {
     const int32_t c0 = cta_of_unit(M.ubeg, r.grid, r.total_units);
@@ -859,22 +859,22 @@ __global__ void __launch_bounds__(kMergeThreads, 2) merge_kernel(const __grid_co
   const int64_t pairs = (static_cast<int64_t>(a.T) + 1) / 2;  // tenants go in twos
   const int64_t t0 = 2 * (pairs * chunk / a.chunks), t1 = min(static_cast<int64_t>(a.T), 2 * (pairs * (chunk + 1) / a.chunks));
   const int32_t* blkptr = table<int32_t>(a.plan, a.off_blkptr) + g * a.Gn + h0;
-  const int eg0 = __ldg(blkptr), ne = __ldg(blkptr + (h1 - h0)) - eg0;
-  for (int x = threadIdx.x; x <= h1 - h0; x += kMergeThreads) ptr_s[x] = __ldg(blkptr + x) - eg0;
+  const int eg0 = ld_g(blkptr), ne = ld_g(blkptr + (h1 - h0)) - eg0;
+  for (int x = threadIdx.x; x <= h1 - h0; x += kMergeThreads) ptr_s[x] = ld_g(blkptr + x) - eg0;
   const bool staged = ne <= kMergeEnt;
   const int tb = staged ? (ne > 0 ? min(static_cast<int64_t>(kMergeVal / ne), t1 - t0) : t1 - t0) : t1 - t0;  // tenants per batch
   if (staged) {
     for (int e = threadIdx.x; e < ne; e += kMergeThreads) {
-      const int2 en = __ldg(blkent + eg0 + e);
+      const int2 en = ld_g(blkent + eg0 + e);
       ent_s[e] = en.x;
       q_s[e] = en.y;
     }
   }
   for (int idx = threadIdx.x; idx < 1024; idx += kMergeThreads) {
     const int w = idx & 31, x = idx >> 5, i = x >> 1, s = x & 1;  // column x = 2i + s of the group block, row w
-    const float o = 4.f * __ldg(a.fout_val + 32 * (i * a.rho_out + s) + w);
+    const float o = 4.f * ld_g(a.fout_val + 32 * (i * a.rho_out + s) + w);
     Dout2[x][w] = make_float2(o, o);
-    DinT[x][w] = 4.f * __ldg(a.fin_val + 32 * (i * a.rho_in + s) + w);
+    DinT[x][w] = 4.f * ld_g(a.fin_val + 32 * (i * a.rho_in + s) + w);
   }
   const Elem* W0 = static_cast<const Elem*>(a.W0) + static_cast<int64_t>(32 * g + rl) * a.ldw + cl * PER;
   const int64_t tstride = static_cast<int64_t>(a.m) * a.ldw;
@@ -885,7 +885,7 @@ __global__ void __launch_bounds__(kMergeThreads, 2) merge_kernel(const __grid_co
     if (staged) {
       for (int x = threadIdx.x; x < nt * ne; x += kMergeThreads) {
         const int t = x / ne, e = x - t * ne;
-        cv_s[x] = __ldg(a.c_vals + (tb0 + t) * a.nnz + q_s[e]);
+        cv_s[x] = ld_g(a.c_vals + (tb0 + t) * a.nnz + q_s[e]);
       }
     }
     __syncthreads();
@@ -895,7 +895,7 @@ __global__ void __launch_bounds__(kMergeThreads, 2) merge_kernel(const __grid_co
 #pragma unroll
       for (int r = 0; r < PASSES; ++r) {
         float w[PER];
-        IO::unpack(__ldg(reinterpret_cast<const uint4*>(W0 + static_cast<int64_t>(r * RPP) * a.ldw + 32 * hb)), w);
+        IO::unpack(ld_g(reinterpret_cast<const uint4*>(W0 + static_cast<int64_t>(r * RPP) * a.ldw + 32 * hb)), w);
 #pragma unroll
         for (int j = 0; j < PER / 2; ++j) w0[r][j] = f2_pack(w[2 * j], w[2 * j + 1]);
       }
@@ -917,10 +917,10 @@ __global__ void __launch_bounds__(kMergeThreads, 2) merge_kernel(const __grid_co
 #pragma unroll
             for (int k = 0; k < TT; ++k) c[k] = cv_s[(t + k) * ne + e];
           } else {
-            const int2 en = __ldg(blkent + eg0 + e);
+            const int2 en = ld_g(blkent + eg0 + e);
             ex = en.x;
 #pragma unroll
-            for (int k = 0; k < TT; ++k) c[k] = __ldg(a.c_vals + (tb0 + t + k) * a.nnz + en.y);
+            for (int k = 0; k < TT; ++k) c[k] = ld_g(a.c_vals + (tb0 + t + k) * a.nnz + en.y);
           }
           const int al = ex & 31, bl = (ex >> 8) & 31;
           uint64_t din[PER / 2];
@@ -1003,7 +1003,7 @@ __global__ void __launch_bounds__(256) adamw_kernel(const AdamWK a) {
     const int64_t n4 = a.n >> 2;
     for (int64_t i = i0; i < n4; i += stride) {
       float4 p = reinterpret_cast<const float4*>(a.p)[i];
-      const float4 g = __ldg(reinterpret_cast<const float4*>(a.g) + i);
+      const float4 g = ld_g(reinterpret_cast<const float4*>(a.g) + i);
       float4 m = reinterpret_cast<const float4*>(a.m)[i];
       float4 v = reinterpret_cast<const float4*>(a.v)[i];
       adamw_one(p.x, g.x, m.x, v.x, a);
@@ -1014,9 +1014,9 @@ __global__ void __launch_bounds__(256) adamw_kernel(const AdamWK a) {
       reinterpret_cast<float4*>(a.m)[i] = m;
       reinterpret_cast<float4*>(a.v)[i] = v;
     }
-    for (int64_t i = (n4 << 2) + i0; i < a.n; i += stride) adamw_one(a.p[i], __ldg(a.g + i), a.m[i], a.v[i], a);
+    for (int64_t i = (n4 << 2) + i0; i < a.n; i += stride) adamw_one(a.p[i], ld_g(a.g + i), a.m[i], a.v[i], a);
   } else {
-    for (int64_t i = i0; i < a.n; i += stride) adamw_one(a.p[i], __ldg(a.g + i), a.m[i], a.v[i], a);
+    for (int64_t i = i0; i < a.n; i += stride) adamw_one(a.p[i], ld_g(a.g + i), a.m[i], a.v[i], a);
   }
 }
 

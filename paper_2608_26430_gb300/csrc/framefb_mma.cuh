@@ -58,7 +58,7 @@ __device__ __forceinline__ void mma_tf32(float (&c)[4], uint32_t a0, uint32_t a1
 // 4 x the group-0 block of a k = 16 frame: D4[w][x], coordinate w of the
 // group, coefficient x = 2i + s <-> frame column i*rho + s.
 __device__ __forceinline__ float d4(const float* val, int rho, int w, int x) {
-  return 4.f * __ldg(val + 32 * ((x >> 1) * rho + (x & 1)) + w);
+  return 4.f * ld_g(val + 32 * ((x >> 1) * rho + (x & 1)) + w);
 }
 
 // Slot permutations (see file comment).  Analysis: K slot k = 16s + 8h + 2t + e

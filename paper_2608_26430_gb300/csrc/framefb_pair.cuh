@@ -152,18 +152,18 @@ __device__ __forceinline__ void load_share(Share<KE>& ch, uint8_t* sp, int mode,
     float zc = 0.f, gc = 0.f;
     const int ez = half * ch.hZ + i, eg = half * ch.hG + i;
     if (i < ch.hZ && ez < h.EZ) {
-      zw = word(static_cast<uint32_t>(__ldg(tab(h.off_zb) + ez * kColumns + col)), 0, 1);
-      const int32_t qi = __ldg(tab(h.off_zq) + ez * kColumns + col);
-      zc = qi >= 0 ? __ldg(c_val + qi) : 0.f;
+      zw = word(static_cast<uint32_t>(ld_g(tab(h.off_zb) + ez * kColumns + col)), 0, 1);
+      const int32_t qi = ld_g(tab(h.off_zq) + ez * kColumns + col);
+      zc = qi >= 0 ? ld_g(c_val + qi) : 0.f;
       const uint32_t tg = zw >> 16;
       openZ = qi >= 0 && tg == FFB_NO_STORE;
       if (firstZ == FFB_NO_STORE) firstZ = tg;
     }
     if (i < ch.hG && eg < h.EG) {
-      gw = word(static_cast<uint32_t>(__ldg(tab(h.off_ga) + eg * kColumns + col)), 1, 0);
-      gb = 8u * slot(0, static_cast<uint32_t>(__ldg(tab(h.off_gb) + eg * kColumns + col)));
-      const int32_t qi = __ldg(tab(h.off_gq) + eg * kColumns + col);
-      gc = (D && qi >= 0) ? __ldg(c_val + qi) : 0.f;
+      gw = word(static_cast<uint32_t>(ld_g(tab(h.off_ga) + eg * kColumns + col)), 1, 0);
+      gb = 8u * slot(0, static_cast<uint32_t>(ld_g(tab(h.off_gb) + eg * kColumns + col)));
+      const int32_t qi = ld_g(tab(h.off_gq) + eg * kColumns + col);
+      gc = (D && qi >= 0) ? ld_g(c_val + qi) : 0.f;
       const uint32_t tg = gw >> 16;
       openG = qi >= 0 && tg == FFB_NO_STORE;
       if (!D) gw |= FFB_NO_STORE << 16;
@@ -297,7 +297,7 @@ __device__ __forceinline__ void fix_runs(const uint8_t* plan, int nfZ, int nfix,
   for (int w = threadIdx.x; w < nfix * npair; w += NT) {
     const int p = w / nfix, i = w - p * nfix;
     const bool z = i < nfZ;
-    const int4 it = z ? __ldg(fz + i) : __ldg(fg + (i - nfZ));
+    const int4 it = z ? ld_g(fz + i) : ld_g(fg + (i - nfZ));
     float2* R = (z ? RZ : RG) + p * pair;
     const uint32_t dst = slot(z ? 1 : 0, static_cast<uint32_t>(it.x));
     float2 a = R[dst];
@@ -319,7 +319,7 @@ __device__ __forceinline__ void flush_dc(const uint8_t* plan, float* dst, const 
   for (int i = 0; i < KE; ++i) {
     const int e = half * hG + i;
     if (i < hG && e < h.EG) {
-      const int32_t qi = __ldg(gq + e * kColumns + col);
+      const int32_t qi = ld_g(gq + e * kColumns + col);
       if (qi >= 0) dst[qi] = dc[i];
     }
   }

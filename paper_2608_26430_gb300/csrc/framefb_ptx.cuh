@@ -144,6 +144,31 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
   for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+// A global load of a kernel launched by launch_chained, of a value that the kernel
+// itself does not write.  Not the read-only form (__ldg): that says that the value
+// does not change while the kernel lives, and such a kernel lives from before the
+// one ahead of it has written its results (C after an optimiser step, dC, the
+// activations), so the compiler could move the load above chain_wait().  Volatile
+// statements keep their order, and the compiler schedules them as it did __ldg
+// (plain loads, which it keeps in order with stores, spilled in group_kernel).
+template <typename T>
+__device__ __forceinline__ T ld_g(const T* p) {
+  static_assert(sizeof(T) == 4 || sizeof(T) == 8 || sizeof(T) == 16, "one load");
+  union {
+    uint32_t w[sizeof(T) / 4];
+    T v;
+  } u;
+  if constexpr (sizeof(T) == 4)
+    asm volatile("ld.global.u32 %0, [%1];" : "=r"(u.w[0]) : "l"(p));
+  else if constexpr (sizeof(T) == 8)
+    asm volatile("ld.global.v2.u32 {%0, %1}, [%2];" : "=r"(u.w[0]), "=r"(u.w[1]) : "l"(p));
+  else
+    asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(u.w[0]), "=r"(u.w[1]), "=r"(u.w[2]), "=r"(u.w[3])
+                 : "l"(p));
+  return u.v;
+}
+
 // Start of a kernel launched by launch_chained (framefb_launch.h): waits until
 // the kernels ahead on the stream have ended and their writes are visible.
 // First statement of such a kernel: nothing reads or writes memory before it.

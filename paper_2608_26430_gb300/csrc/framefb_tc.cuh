@@ -71,7 +71,7 @@ __device__ __forceinline__ void dc_flush(const uint8_t* plan, float* dst, const 
 #pragma unroll
   for (int e = 0; e < KE; ++e) {
     if (e < h.EG) {
-      const int32_t q = __ldg(gq + e * kThreads + col);
+      const int32_t q = ld_g(gq + e * kThreads + col);
       if (q >= 0) dst[q] = dc[e];
     }
   }
@@ -265,17 +265,17 @@ __device__ __forceinline__ void tc_load_chunk(Chunk<MODE, true, false>& ch, cons
     ch.gb[e] = 0;
     ch.zc[e] = ch.gc[e] = 0.f;
     if (F && e < ch.EZ) {
-      const uint32_t w = static_cast<uint32_t>(__ldg(tzb + e * kThreads + col));
+      const uint32_t w = static_cast<uint32_t>(ld_g(tzb + e * kThreads + col));
       ch.zb[e] = slots(w, ch.n, ch.m);
-      const int32_t q = __ldg(tzq + e * kThreads + col);
-      ch.zc[e] = q >= 0 ? __ldg(c_val + q) : 0.f;
+      const int32_t q = ld_g(tzq + e * kThreads + col);
+      ch.zc[e] = q >= 0 ? ld_g(c_val + q) : 0.f;
     }
     if ((D || C) && e < ch.EG) {
-      const uint32_t w = static_cast<uint32_t>(__ldg(tga + e * kThreads + col));
+      const uint32_t w = static_cast<uint32_t>(ld_g(tga + e * kThreads + col));
       ch.ga[e] = slots(w, ch.m, ch.n);
-      ch.gb[e] = static_cast<uint32_t>(tc_slot(__ldg(tgb + e * kThreads + col), ch.n));
-      const int32_t q = __ldg(tgq + e * kThreads + col);
-      ch.gc[e] = (D && q >= 0) ? __ldg(c_val + q) : 0.f;
+      ch.gb[e] = static_cast<uint32_t>(tc_slot(ld_g(tgb + e * kThreads + col), ch.n));
+      const int32_t q = ld_g(tgq + e * kThreads + col);
+      ch.gc[e] = (D && q >= 0) ? ld_g(c_val + q) : 0.f;
     }
   }
 }
@@ -453,8 +453,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_tile_kernel(const __grid_con
 #pragma unroll
       for (int mt = 0; mt < kTcMaxTiles; ++mt) {
         const int r = r0 + 128 * mt;
-        on_y[mt] = F && r < h.Gm && __ldg(zm + r) != 0u;
-        on_x[mt] = D && r < h.Gn && __ldg(gm + r) != 0u;
+        on_y[mt] = F && r < h.Gm && ld_g(zm + r) != 0u;
+        on_x[mt] = D && r < h.Gn && ld_g(gm + r) != 0u;
       }
     };
     for (int s = 0; s < count + 2; ++s) {
@@ -625,8 +625,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_tile_kernel(const __grid_con
             nfZ = F ? h.nfixZ : 0;
             nfix = nfZ + (D ? h.nfixG : 0);
             for (int i = st; i < nfix; i += kTcSpmm)
-              fixc[i] = i < nfZ ? __ldg(table<int4>(splan, h.off_fixZ) + i)
-                                : __ldg(table<int4>(splan, h.off_fixG) + (i - nfZ));
+              fixc[i] = i < nfZ ? ld_g(table<int4>(splan, h.off_fixZ) + i)
+                                : ld_g(table<int4>(splan, h.off_fixG) + (i - nfZ));
             tc_spmm_bar();
           }
         }

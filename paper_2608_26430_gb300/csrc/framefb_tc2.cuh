@@ -144,17 +144,17 @@ __device__ __forceinline__ void tc2_load_chunk(Chunk<MODE, true, false>& ch, con
     ch.gb[e] = 0;
     ch.zc[e] = ch.gc[e] = 0.f;
     if (F && e < ch.EZ) {
-      const uint32_t w = static_cast<uint32_t>(__ldg(tzb + e * kThreads + col));
+      const uint32_t w = static_cast<uint32_t>(ld_g(tzb + e * kThreads + col));
       ch.zb[e] = offsets(w, ch.m);
-      const int32_t q = __ldg(tzq + e * kThreads + col);
-      ch.zc[e] = q >= 0 ? __ldg(c_val + q) : 0.f;
+      const int32_t q = ld_g(tzq + e * kThreads + col);
+      ch.zc[e] = q >= 0 ? ld_g(c_val + q) : 0.f;
     }
     if ((D || C) && e < ch.EG) {
-      const uint32_t w = static_cast<uint32_t>(__ldg(tga + e * kThreads + col));
+      const uint32_t w = static_cast<uint32_t>(ld_g(tga + e * kThreads + col));
       ch.ga[e] = offsets(w, ch.n);
-      ch.gb[e] = 8u * static_cast<uint32_t>(vu_slot(__ldg(tgb + e * kThreads + col)));
-      const int32_t q = __ldg(tgq + e * kThreads + col);
-      ch.gc[e] = (D && q >= 0) ? __ldg(c_val + q) : 0.f;
+      ch.gb[e] = 8u * static_cast<uint32_t>(vu_slot(ld_g(tgb + e * kThreads + col)));
+      const int32_t q = ld_g(tgq + e * kThreads + col);
+      ch.gc[e] = (D && q >= 0) ? ld_g(c_val + q) : 0.f;
     }
   }
 }
@@ -304,8 +304,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc2_tile_kernel(const __grid_co
       wide_x = (reinterpret_cast<uintptr_t>(X2) & 31u) == 0 && (ldx2 & 15) == 0;
       const uint8_t* plan = args.m[j].plan;
       const FfbPlanHeader& h = hdr(plan);
-      on_y = F && r0 < Gm2 && __ldg(table<uint32_t>(plan, h.off_zmask) + r0) != 0u;
-      on_x = D && r0 < Gn2 && __ldg(table<uint32_t>(plan, h.off_gmask) + r0) != 0u;
+      on_y = F && r0 < Gm2 && ld_g(table<uint32_t>(plan, h.off_zmask) + r0) != 0u;
+      on_x = D && r0 < Gn2 && ld_g(table<uint32_t>(plan, h.off_gmask) + r0) != 0u;
     };
     for (int s = 0; s < count + 2; ++s) {
       const int i2 = s - 2, i1 = s - 1;
@@ -503,8 +503,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc2_tile_kernel(const __grid_co
             nfZ = F ? h.nfixZ : 0;
             nfix = nfZ + (D ? h.nfixG : 0);
             for (int i = st; i < nfix; i += kTcSpmm)
-              fixc[i] = i < nfZ ? __ldg(table<int4>(splan, h.off_fixZ) + i)
-                                : __ldg(table<int4>(splan, h.off_fixG) + (i - nfZ));
+              fixc[i] = i < nfZ ? ld_g(table<int4>(splan, h.off_fixZ) + i)
+                                : ld_g(table<int4>(splan, h.off_fixG) + (i - nfZ));
           }
         }
       }

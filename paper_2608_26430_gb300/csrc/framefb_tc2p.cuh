@@ -178,8 +178,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc2p_tile_kernel(const __grid_c
       wide_x = (reinterpret_cast<uintptr_t>(X2) & 31u) == 0 && (ldx2 & 15) == 0;
       const uint8_t* plan = args.m[j].plan;
       const FfbPlanHeader& h = hdr(plan);
-      on_y = F && py < P2 && __ldg(table<uint32_t>(plan, h.off_zmask) + gy) != 0u;
-      on_x = D && px < P2 && __ldg(table<uint32_t>(plan, h.off_gmask) + gx) != 0u;
+      on_y = F && py < P2 && ld_g(table<uint32_t>(plan, h.off_zmask) + gy) != 0u;
+      on_x = D && px < P2 && ld_g(table<uint32_t>(plan, h.off_gmask) + gx) != 0u;
     };
     for (int s = 0; s < count + 2; ++s) {
       const int i2 = s - 2, i1 = s - 1;
@@ -389,8 +389,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc2p_tile_kernel(const __grid_c
             nfZ = F ? h.nfixZ : 0;
             nfix = nfZ + (D ? h.nfixG : 0);
             for (int i = st; i < nfix; i += kTcSpmm)
-              fixc[i] = i < nfZ ? __ldg(table<int4>(splan, h.off_fixZ) + i)
-                                : __ldg(table<int4>(splan, h.off_fixG) + (i - nfZ));
+              fixc[i] = i < nfZ ? ld_g(table<int4>(splan, h.off_fixZ) + i)
+                                : ld_g(table<int4>(splan, h.off_fixG) + (i - nfZ));
           }
         }
       }
