@@ -735,6 +735,30 @@ bool parts_allowed() {
   return !(e && std::strcmp(e, "0") == 0);
 }
 
+// The group-transform kernel (framefb_grp.cu) runs the matrix.  bf16 plans that
+// the fused tcgen05 kernels take whole stay with them (a forward pass there needs
+// no workspace), and so do calls without dX over a plan of parts that has at most
+// 16 entries per column: one part per block of outputs then, in one launch, and
+// every output is written once.  One matrix, 4096 entries, this kernel against
+// those routes, us at 128 / 1024 / 4096 tokens:
+//   8192 -> 4096, forward: 14 / 28 / 74 against 12 / 20 / 51 (Zipf rows
+//     16 / 35 / 95, 12 / 23 / 63)
+//   1024 -> 8192, fused pass: 25 / 53 / 142 against 30 / 47 / 110
+//   8192 -> 8192, fused pass: 30 / 64 / 168 against 40 / 72 / 189, but 103 and 81
+//     on a forward pass of 4096 tokens (Zipf rows)
+//   4096 -> 14336, forward: 17 / 36 / 104 against 11 / 30 / 102, dC alone
+//     22 / 44 / 106 against 19 / 35 / 95; with dX the parts take turns, fused pass
+//     32 / 71 / 188 against 91 / 140 / 300.
+bool group_route(const framefb_mat& M, const FfbPlanHeader& h, int32_t ops, framefb_dtype dt) {
+  if (!tc_allowed()) return false;
+  if (dt == FRAMEFB_BF16) {
+    if (fused_tc_ok(h)) return false;
+    const bool short_columns = h.EZ <= ffb::kEreg && h.EG <= ffb::kEreg;
+    if (!(ops & FRAMEFB_OP_BACKWARD_DX) && short_columns && parts_allowed() && !M.plan->subs.empty()) return false;
+  }
+  return ffb_host::grp_takes(M, ops, dt);
+}
+
 // Matrices of a call split by path, each in call order: the row-transform
 // kernel (framefb_row.cu), the fused kernels
 // (structured plans they take, fp32, or rows with padding), the plans' parts
@@ -757,7 +781,7 @@ framefb_status split_paths(const framefb_mat* mats, int32_t nmats, int32_t ops, 
         row.push_back(M);
         continue;
       }
-      if (tc_allowed() && ffb_host::grp_takes(M, ops, dt)) {
+      if (group_route(M, *h, ops, dt)) {
         fft.push_back(M);
         continue;
       }

@@ -1,0 +1,72 @@
+"""Which kernels a call runs on, and what it needs, at the lines between the
+routes of structured plans (checked against the fp64 oracle: bf16 bar for Y and
+dX, 1e-5 relative for fp32)."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from paper_2608_26430_gb300 import framefb as ffb
+from paper_2608_26430_gb300 import workloads as wl
+from paper_2608_26430_gb300.batch import AdapterBatch
+from tests.oracle_side import Expect, assert_bf16, host64
+
+pytestmark = pytest.mark.gpu
+
+DEV = "cuda:0"
+F, ALL = ffb.OP_FORWARD, ffb.OP_FORWARD | ffb.OP_BACKWARD_DX | ffb.OP_GRAD_COEFF
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2608_26430_gb300.build import build
+    build()
+    ffb.lib()
+
+
+def load(mats, N, nnz, dtype="bf16", **kw):
+    return wl.Workload("routes", tuple(wl.MatSpec(f"w{i}", n, m) for i, (n, m) in enumerate(mats)), N=N, nnz=nnz,
+                       dtype=dtype, c_std=0.02, **kw)
+
+
+def names(b, ops):
+    return ffb.framefb_kernel_names(b.mats, ops, b.dtype_code)
+
+
+# sides of up to 256 groups, at most 16 entries per column: whole on the fused
+# tcgen05 kernels at any token count, a forward pass without a workspace
+@pytest.mark.parametrize("shape", [(8192, 1024), (1024, 8192), (8192, 8192)])
+@pytest.mark.parametrize("N", [5, 131])
+def test_wide_sides_of_the_fused_kernels(shape, N):
+    b = AdapterBatch(load([shape], N, 900), DEV, ops=ALL)
+    assert names(b, F) == ["tc_tile_kernel<1>"]
+    assert ffb.framefb_workspace_size(b.mats, F) == 0
+    ffb.framefb_forward(b.mats, b.dtype_code, None)
+    e, buf = Expect(b, 0), b.bufs[0]
+    X = host64(buf.X)
+    torch.cuda.synchronize()
+    assert_bf16(host64(buf.Y), e.y(X, np.zeros((N, shape[1]))), what="Y")
+    buf.Y.zero_()
+    vals = torch.stack([buf.c_val, 2 * buf.c_val])
+    m = ffb.framefb_mat.from_buffer_copy(b.mats[0])
+    m.c_val = vals.data_ptr()
+    ffb.framefb_forward_tenants([m], b.dtype_code, [0, 2, N], [1, 0], 2)
+    torch.cuda.synchronize()
+    want = e.y(X, np.zeros((N, shape[1])))
+    want[:2] *= 2
+    assert_bf16(host64(buf.Y), want, what="Y of tenants")
+
+
+@pytest.mark.parametrize("ops", [F, ffb.OP_GRAD_COEFF])
+def test_parts_of_short_columns_without_dx(ops):
+    b = AdapterBatch(load([(1024, 9216)], 37, 700), DEV, ops=ops)
+    assert names(b, ops) == [f"tc2_tile_kernel<{ops}>"]
+    b.run(ops, b.workspace(ops))
+    torch.cuda.synchronize()
+    e, buf = Expect(b, 0), b.bufs[0]
+    if ops == F:
+        assert_bf16(host64(buf.Y), e.y(host64(buf.X), np.zeros((37, 9216))), what="Y")
+    else:
+        assert_bf16(host64(buf.dC), e.dc(host64(buf.X), host64(buf.dY)), what="dC")
