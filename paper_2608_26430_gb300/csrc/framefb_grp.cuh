@@ -257,8 +257,8 @@ __device__ __forceinline__ void load_cols(Cols& ch, uint8_t* sp, int mode, const
   const bool F = mode & kF, D = mode & kD, C = mode & kC;
   const FfbPlanHeader& h = *reinterpret_cast<const FfbPlanHeader*>(plan);
   auto tab = [&](int32_t off) { return reinterpret_cast<const int32_t*>(plan + off); };
-  ch.hZ = F ? (h.EZ + H - 1) / H : 0;
-  ch.hG = D || C ? (h.EG + H - 1) / H : 0;
+  ch.hZ = F ? half_of<H>(h.EZ) : 0;
+  ch.hG = D || C ? half_of<H>(h.EG) : 0;
   const int K[2] = {h.n, h.m};
   auto word = [&](uint32_t w, int ts) {  // store target of side ts
     const uint32_t t = w >> 16;
@@ -402,8 +402,8 @@ __device__ __forceinline__ void load_big(Big& ch, uint8_t* sp, int mode, const u
   const bool F = mode & kF, D = mode & kD, C = mode & kC;
   const FfbPlanHeader& h = *reinterpret_cast<const FfbPlanHeader*>(plan);
   auto tab = [&](int32_t off) { return reinterpret_cast<const int32_t*>(plan + off); };
-  ch.hZ = F ? (h.EZ + 1) / 2 : 0;
-  ch.hG = D || C ? (h.EG + 1) / 2 : 0;
+  ch.hZ = F ? half_of<2>(h.EZ) : 0;
+  ch.hG = D || C ? half_of<2>(h.EG) : 0;
   const int K[2] = {h.n, h.m};
   auto target = [&](uint32_t t, int sd) {
     return static_cast<int>(t) < K[sd] ? slot(sd, t) : over(sd, t - K[sd]);

@@ -124,6 +124,16 @@ __device__ __forceinline__ void get_plan(const uint8_t* sp, int a, int i0, uint3
   v[3] = x.w;
 }
 
+// Entries per thread of a column of E entries with H threads per column.  With
+// two, the first takes whole blocks of four: the loops walk blocks, and an entry
+// past its share, inside the block, would add 0 x (the gathered value) to the run
+// that it passes on to the second half, which is not 0 for an infinity or a NaN.
+// (Entries past the end of a column follow its last store and reach nothing.)
+template <int H>
+__device__ __forceinline__ int half_of(int E) {
+  return H == 2 ? ((E + 1) / 2 + 3) & ~3 : E;
+}
+
 // slot(side, x): index of frame column x of a side (0 input, 1 output) in its
 // buffers (float2); overflow slots (x >= the side's columns) stay as they are.
 template <int KE, int H, int NT, typename Slot>
@@ -132,8 +142,8 @@ __device__ __forceinline__ void load_share(Share<KE>& ch, uint8_t* sp, int mode,
   const bool F = mode & kF, D = mode & kD, C = mode & kC;
   const FfbPlanHeader& h = *reinterpret_cast<const FfbPlanHeader*>(plan);
   auto tab = [&](int32_t off) { return reinterpret_cast<const int32_t*>(plan + off); };
-  ch.hZ = F ? (h.EZ + H - 1) / H : 0;
-  ch.hG = D || C ? (h.EG + H - 1) / H : 0;
+  ch.hZ = F ? half_of<H>(h.EZ) : 0;
+  ch.hG = D || C ? half_of<H>(h.EG) : 0;
   const int K[2] = {h.n, h.m};
   // gather index of side sd | store target of side ts << 16
   auto word = [&](uint32_t w, int sd, int ts) {
