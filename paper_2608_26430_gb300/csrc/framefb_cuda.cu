@@ -749,25 +749,28 @@ bool parts_allowed() {
 //   4096 -> 14336, forward: 17 / 36 / 104 against 11 / 30 / 102, dC alone
 //     22 / 44 / 106 against 19 / 35 / 95; with dX the parts take turns, fused pass
 //     32 / 71 / 188 against 91 / 140 / 300.
+// (FRAMEFB_PARTS=0 leaves the other bf16 plans to the contraction path.)
 bool group_route(const framefb_mat& M, const FfbPlanHeader& h, int32_t ops, framefb_dtype dt) {
   if (!tc_allowed()) return false;
   if (dt == FRAMEFB_BF16) {
-    if (fused_tc_ok(h)) return false;
+    if (fused_tc_ok(h) || !parts_allowed()) return false;
     const bool short_columns = h.EZ <= ffb::kEreg && h.EG <= ffb::kEreg;
-    if (!(ops & FRAMEFB_OP_BACKWARD_DX) && short_columns && parts_allowed() && !M.plan->subs.empty()) return false;
+    if (!(ops & FRAMEFB_OP_BACKWARD_DX) && short_columns && !M.plan->subs.empty()) return false;
   }
   return ffb_host::grp_takes(M, ops, dt);
 }
 
 // Matrices of a call split by path, each in call order: the row-transform
-// kernel (framefb_row.cu), the fused kernels
-// (structured plans they take, fp32, or rows with padding), the plans' parts
-// on the fused tcgen05 kernels (bf16 structured plans the kernels do not
-// take whole, with parts, and tokens; FRAMEFB_PARTS=0 sends them to the
-// contraction path), and the contraction path of framefb_dense.cu
-// (dense-layout plans, and the other bf16 structured plans the fused
-// tcgen05 kernels do not take, with unpadded rows).  FRAMEFB_KERNEL=tile
-// keeps every structured plan on the warp-MMA kernel.
+// kernel (framefb_row.cu), the group-transform kernel (framefb_grp.cu: fp32, and
+// wide bf16 plans, group_route), the fused kernels (structured plans they take,
+// fp32 plans too large for the group transform, or rows with padding), the
+// plans' parts on the fused tcgen05 kernels (the other bf16 structured plans with
+// parts, and tokens), and the contraction path of framefb_dense.cu (dense-layout
+// plans the row transform does not take, and what is left of the bf16
+// structured plans, with unpadded rows).  FRAMEFB_PARTS=0 sends every bf16
+// structured plan that the fused tcgen05 kernels do not take whole to the
+// contraction path; FRAMEFB_KERNEL=tile keeps every structured plan on the
+// warp-MMA kernel (bf16) or the one-phase FFT kernel (fp32).
 framefb_status split_paths(const framefb_mat* mats, int32_t nmats, int32_t ops, framefb_dtype dt,
                            std::vector<framefb_mat>& grp, std::vector<framefb_mat>& den, std::vector<framefb_mat>& row,
                            std::vector<framefb_mat>& fft,

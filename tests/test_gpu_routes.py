@@ -70,3 +70,18 @@ def test_parts_of_short_columns_without_dx(ops):
         assert_bf16(host64(buf.Y), e.y(host64(buf.X), np.zeros((37, 9216))), what="Y")
     else:
         assert_bf16(host64(buf.dC), e.dc(host64(buf.X), host64(buf.dY)), what="dC")
+
+
+@pytest.mark.parametrize("shape,N", [((1024, 4608), 45), ((4608, 1024), 200)])
+def test_without_parts_wide_plans_run_as_contractions(shape, N, monkeypatch):
+    monkeypatch.setenv("FRAMEFB_PARTS", "0")
+    b = AdapterBatch(load([shape], N, 4300, support_mode=wl.ZIPF_ROWS), DEV, ops=ALL)
+    assert "dense_gemm_kernel<bf16_hilo><grouped>" in names(b, ALL)
+    assert all(k.startswith(("dense_", "group_block_kernel")) for k in names(b, ALL))
+    b.run(ALL, b.workspace(ALL))
+    torch.cuda.synchronize()
+    e, buf = Expect(b, 0), b.bufs[0]
+    X, dY = host64(buf.X), host64(buf.dY)
+    assert_bf16(host64(buf.Y), e.y(X, np.zeros((N, shape[1]))), what="Y")
+    assert_bf16(host64(buf.dX), e.dx(dY, np.zeros((N, shape[0]))), what="dX")
+    assert_bf16(host64(buf.dC), e.dc(X, dY), what="dC")
