@@ -390,8 +390,8 @@ def time_config(name, dev, stream, steps, warmup, flush, with_cpu, headline=None
     rec = {"ms_per_step": ms, "tokens_per_s": w.N / (ms / 1e3), "matrices": len(w.mats), "tokens": w.N,
            "dtype": w.dtype, "algorithmic_bytes": alg, "achieved_gbs": gbs, "frac_of_measured": gbs / peak,
            "frac_of_8tbs": gbs / NOMINAL_GBS,
-           "kernels": kernels + (["dc_reduce_kernel"] if any(k.startswith(("tc", "mma")) for k in kernels) else [])
-           + (["pair_reduce_kernel"] if any(k.startswith(("row", "fft")) for k in kernels) else []),
+           "kernels": kernels + (["dc_reduce_kernel"] if any(k.startswith(("tc", "mma", "fft_phase")) for k in kernels) else [])
+           + (["pair_reduce_kernel"] if any(k.startswith(("row", "fft_tile")) for k in kernels) else []),
            "l2": "L2 flushed between steps" if alg < 2 * L2_BYTES else "step moves more than L2"}
     if flops:
         tpk, kind = tensor_peak()

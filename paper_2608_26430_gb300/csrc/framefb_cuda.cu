@@ -133,7 +133,7 @@ void* tile_kernel_ptr(framefb_dtype dt, int mode, bool reg, int T) {
                          : reinterpret_cast<void*>(ffb::mma_tile_kernel<M, false, 1>));
 #define FFB_FFT(M) \
   case M:          \
-    return reg ? reinterpret_cast<void*>(ffb::fft_tile_kernel<M, true>) : reinterpret_cast<void*>(ffb::fft_tile_kernel<M, false>);
+    return reg ? reinterpret_cast<void*>(ffb::fft_phase_kernel<M, true>) : reinterpret_cast<void*>(ffb::fft_phase_kernel<M, false>);
   if (dt == FRAMEFB_BF16) {
     if (T != 1 && T != 2) return nullptr;
     switch (mode) {
@@ -715,7 +715,7 @@ framefb_status structured_names(const framefb_mat* mats, int32_t nmats, int32_t 
     std::string k = P.pack  ? "tc2p_tile_kernel"
                     : P.tc2 ? "tc2_tile_kernel"
                     : P.tc  ? "tc_tile_kernel"
-                            : (dtype == FRAMEFB_BF16 ? "mma_tile_kernel" : "fft_tile_kernel");
+                            : (dtype == FRAMEFB_BF16 ? "mma_tile_kernel" : "fft_phase_kernel");
     k += "<" + std::to_string(ops) + ">";
     if (std::find(names.begin(), names.end(), k) == names.end()) names.push_back(k);
   }

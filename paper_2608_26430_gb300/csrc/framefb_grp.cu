@@ -115,8 +115,8 @@ Variant variant(const FfbPlanHeader* h) {
 void* kernel_ptr(const Variant& v, framefb_dtype dt) {
 #define FFB_GRP(N, E, B)                                                                             \
   if (v == Variant{N, E, B})                                                                         \
-    return dt == FRAMEFB_BF16 ? reinterpret_cast<void*>(fg::group_kernel<__nv_bfloat16, N, E, B>)    \
-                              : reinterpret_cast<void*>(fg::group_kernel<float, N, E, B>);
+    return dt == FRAMEFB_BF16 ? reinterpret_cast<void*>(fg::fft_tile_kernel<__nv_bfloat16, N, E, B>)    \
+                              : reinterpret_cast<void*>(fg::fft_tile_kernel<float, N, E, B>);
   FFB_GRP(256, 4, false)
   FFB_GRP(256, 8, false)
   FFB_GRP(512, 8, false)

@@ -518,7 +518,7 @@ __device__ __forceinline__ void spmm_big(const Big& ch, uint8_t* sp, bool F, boo
 
 // ---------------------------------------------------------------------------
 template <typename Elem, int NT, int KE, bool BIG>
-__global__ void __launch_bounds__(NT, NT == 512 ? 1 : 2) group_kernel(const __grid_constant__ Launch args) {
+__global__ void __launch_bounds__(NT, NT == 512 ? 1 : 2) fft_tile_kernel(const __grid_constant__ Launch args) {
   chain_wait();
   chain_next();
   static_assert(!BIG || (NT == 512 && KE == kBigE), "big plans: two threads per column");

@@ -1,4 +1,4 @@
-// Device code of libframefb: the batched tile kernel (S3-S6), the dC
+// Device code of libframefb: the one-phase-at-a-time FFT kernel (S3-S6), the dC
 // reduction and the merge kernel (S7).  Included by framefb_cuda.cu only.
 //
 // The frames of the GPU path have k = 16 and k*rho = d (every config of the
@@ -12,8 +12,9 @@
 // The 1/4 of each side is folded into one scale s/16 applied at the end.
 // The twiddles are read from the caller's device frame (column rho: subspace
 // 1 of group 0 holds omega^j / 4 on coordinates 2j, 2j+1).  This exact FFT
-// serves fp32 activations; bf16 activations use the tensor-core kernel of
-// framefb_mma.cuh.
+// serves the fp32 plans that fft_tile_kernel (framefb_grp.cuh) does not take (more
+// than 32 entries per column, or too large for its buffers), and every fp32 plan
+// under FRAMEFB_KERNEL=tile.
 #pragma once
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -608,7 +609,7 @@ __device__ __forceinline__ int fix_count(const uint8_t* plan, int mode) {
 // workspace slot (cta + matrix) when the CTA leaves the matrix.
 // ---------------------------------------------------------------------------
 template <int MODE, bool REG>
-__global__ void __launch_bounds__(kThreads, 1) fft_tile_kernel(const __grid_constant__ LaunchK args) {
+__global__ void __launch_bounds__(kThreads, 1) fft_phase_kernel(const __grid_constant__ LaunchK args) {
   chain_wait();
   using Elem = float;
   constexpr bool F = MODE & MODE_F, D = MODE & MODE_D, C = MODE & MODE_C;

@@ -150,7 +150,7 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
 // one ahead of it has written its results (C after an optimiser step, dC, the
 // activations), so the compiler could move the load above chain_wait().  Volatile
 // statements keep their order, and the compiler schedules them as it did __ldg
-// (plain loads, which it keeps in order with stores, spilled in group_kernel).
+// (plain loads, which it keeps in order with stores, spilled in fft_tile_kernel).
 template <typename T>
 __device__ __forceinline__ T ld_g(const T* p) {
   static_assert(sizeof(T) == 4 || sizeof(T) == 8 || sizeof(T) == 16, "one load");

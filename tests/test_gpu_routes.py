@@ -9,7 +9,7 @@ torch = pytest.importorskip("torch")
 from paper_2608_26430_gb300 import framefb as ffb
 from paper_2608_26430_gb300 import workloads as wl
 from paper_2608_26430_gb300.batch import AdapterBatch
-from tests.oracle_side import Expect, assert_bf16, host64
+from tests.oracle_side import Expect, assert_bf16, assert_f32, host64
 
 pytestmark = pytest.mark.gpu
 
@@ -85,3 +85,31 @@ def test_without_parts_wide_plans_run_as_contractions(shape, N, monkeypatch):
     assert_bf16(host64(buf.Y), e.y(X, np.zeros((N, shape[1]))), what="Y")
     assert_bf16(host64(buf.dX), e.dx(dY, np.zeros((N, shape[0]))), what="dX")
     assert_bf16(host64(buf.dC), e.dc(X, dY), what="dC")
+
+
+# more than 32 entries per column, or the switch: the one-phase FFT kernel under
+# its own name
+@pytest.mark.parametrize("mats,N,nnz,kernel", [([(256, 256)], 37, 9000, ""), ([(768, 256), (256, 768)], 21, 9000, ""),
+                                               ([(256, 256)] * 3, 9, 200, "tile"), ([(1024, 768)], 33, 4000, "tile")])
+def test_fp32_one_phase_kernel(mats, N, nnz, kernel, monkeypatch):
+    monkeypatch.setenv("FRAMEFB_KERNEL", kernel)
+    b = AdapterBatch(load(mats, N, nnz, "f32"), DEV, ops=ALL)
+    for ops in (F, ffb.OP_BACKWARD_DX, ffb.OP_GRAD_COEFF, ffb.OP_BACKWARD_DX | ffb.OP_GRAD_COEFF, ALL):
+        assert names(b, ops) == [f"fft_phase_kernel<{ops}>"]
+        for x in b.bufs:
+            x.Y.zero_()
+            x.dX.zero_()
+            x.dC.fill_(float("nan"))
+        b.run(ops, b.workspace(ops))
+        torch.cuda.synchronize()
+        for j, x in enumerate(b.bufs):
+            e, X, dY = Expect(b, j), host64(x.X), host64(x.dY)
+            if ops & F:
+                assert_f32(host64(x.Y), e.y(X, np.zeros((N, x.spec.m))), what=f"Y[{j}]")
+            if ops & ffb.OP_BACKWARD_DX:
+                assert_f32(host64(x.dX), e.dx(dY, np.zeros((N, x.spec.n))), what=f"dX[{j}]")
+            if ops & ffb.OP_GRAD_COEFF:
+                assert_f32(host64(x.dC), e.dc(X, dY), what=f"dC[{j}]")
+    monkeypatch.setenv("FRAMEFB_KERNEL", "")
+    if nnz <= 8192:
+        assert names(b, ALL) == ["fft_tile_kernel<7>"]
