@@ -149,32 +149,22 @@ std::vector<Chunk> chunks_of(const framefb_mat* mats, int32_t nmats) {
   }
   std::vector<Chunk> out;
   for (const Variant& v : kinds) {
-    std::vector<const FfbPlanHeader*> shapes;
-    Regions all;  // of one pair of each shape of the chunk
+    Regions all;  // of one pair of each matrix of the chunk
     bool open = false;
+    const framefb_plan* plan = nullptr;
+    fg::Shape sh;
     for (int32_t j = 0; j < nmats; ++j) {
       if (!(of[j] == v)) continue;
-      const FfbPlanHeader* h = header_of(mats[j].plan);
-      bool known = std::find(shapes.begin(), shapes.end(), h) != shapes.end();
-      fg::Shape sh;
+      if (mats[j].plan != plan) shape_of(header_of(plan = mats[j].plan), v, sh);
       Regions with = all;
-      if (!known) {
-        shape_of(h, v, sh);
-        with.take(sh, 1, v);
-      }
-      if (!open || static_cast<int>(out.back().mats.size()) == fg::kMaxMats ||
-          (!known && (static_cast<int>(shapes.size()) == fg::kMaxShapes || with.bytes(v) > budget(v)))) {
+      with.take(sh, 1, v);
+      if (!open || static_cast<int>(out.back().mats.size()) == fg::kMaxMats || with.bytes(v) > budget(v)) {
         out.push_back(Chunk{{}, v});
-        shapes.clear();
-        all = Regions();
+        with = Regions();
+        with.take(sh, 1, v);
         open = true;
-        if (known) shape_of(h, v, sh);
-        known = false;
       }
-      if (!known) {
-        shapes.push_back(h);
-        all.take(sh, 1, v);
-      }
+      all = with;
       out.back().mats.push_back(&mats[j]);
     }
   }
@@ -198,17 +188,19 @@ framefb_status prepare(const Chunk& ch, int32_t ops, framefb_dtype dt, Prepared&
   int64_t pairs = 0;
   for (const framefb_mat* M : ch.mats) pairs += (M->N + 1) / 2;
   const int64_t spread = std::max<int64_t>(1, pairs / (static_cast<int64_t>(sms) * per));
-  std::vector<const FfbPlanHeader*> hd;
   int nsh = 0;
   Regions reg;
   for (int j = 0; j < nm; ++j) {
-    const FfbPlanHeader* h = header_of(ch.mats[j]->plan);
-    const int s = static_cast<int>(std::find(hd.begin(), hd.end(), h) - hd.begin());
+    if (j > 0 && ch.mats[j]->plan == ch.mats[j - 1]->plan) {
+      A.m[j].shape = A.m[j - 1].shape;
+      continue;
+    }
+    fg::Shape sh;
+    if (!shape_of(header_of(ch.mats[j]->plan), ch.v, sh)) return FRAMEFB_EINVAL;
+    int s = 0;  // (plans of one geometry share it)
+    while (s < nsh && std::memcmp(&A.sh[s], &sh, sizeof(sh)) != 0) ++s;
     if (s == nsh) {
-      if (nsh == fg::kMaxShapes) return FRAMEFB_EINVAL;
-      hd.push_back(h);
-      fg::Shape& sh = A.sh[nsh++];
-      if (!shape_of(h, ch.v, sh)) return FRAMEFB_EINVAL;
+      A.sh[nsh++] = sh;
       reg.take(sh, 1, ch.v);
     }
     A.m[j].shape = s;
@@ -261,11 +253,11 @@ framefb_status prepare(const Chunk& ch, int32_t ops, framefb_dtype dt, Prepared&
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, ch.v.nt, P.smem) != cudaSuccess)
     return FRAMEFB_ECUDA;
   if (per_sm < 1) return FRAMEFB_EUNSUPPORTED;
-  // every CTA gets a unit: its share of the cost is at least the largest unit's
-  // (the dC reduction sums the slots of a matrix's first to last CTA)
-  int32_t max_cost = 1;
-  for (int j = 0; j < nm; ++j) max_cost = std::max(max_cost, A.m[j].ntiles > 0 ? A.m[j].cost : 1);
-  P.grid = static_cast<int>(std::min({static_cast<int64_t>(sms) * per_sm, units, A.total_cost / max_cost}));
+  // As many CTAs as there are units, or as are resident.  (With a unit for every
+  // CTA at equal shares, the largest unit's cost bounded the grid: one matrix of
+  // 4096 -> 256 beside two small ones, 64 tokens, forward, then ran on 57 CTAs in
+  // 24.6 us, and the grid fell where more tokens made the units larger.)
+  P.grid = static_cast<int>(std::min<int64_t>(static_cast<int64_t>(sms) * per_sm, units));
   P.ws_bytes = 0;
   if (ops & FRAMEFB_OP_GRAD_COEFF) {
     P.ws_bytes = static_cast<size_t>(P.grid + nm) * A.stride * sizeof(float) + 256;

@@ -36,8 +36,7 @@ namespace grp {
 using namespace pair;
 
 // Bounded by construction: this kernel waits on nothing but CTA barriers.
-constexpr int kMaxShapes = 8;  // distinct geometries of a launch
-constexpr int kMaxMats = 96;   // matrices of a launch
+constexpr int kMaxMats = 96;  // matrices of a launch
 
 // Buffers of a token pair (float2 offsets), side 0 the input side (X, V, RG,
 // dX), side 1 the output side (dY, U, RZ, Y): A[s] V or U, B[s] RG or RZ.
@@ -60,12 +59,26 @@ struct Mat {
   int64_t cbeg;       // cost of the units before ubeg
 };
 
-// First unit of CTA c of `grid`: the units are split at equal cost.
+// Matrix that holds position x of a list whose matrices begin at first(j).
+template <typename First, typename T>
+__host__ __device__ __forceinline__ int32_t matrix_at(int32_t nmats, T x, First first) {
+  int32_t lo = 0, hi = nmats - 1;
+  while (lo < hi) {
+    const int32_t mid = (lo + hi + 1) >> 1;
+    if (first(mid) <= x)
+      lo = mid;
+    else
+      hi = mid - 1;
+  }
+  return lo;
+}
+
+// First unit of CTA c of `grid`: the units are split at equal cost.  (A CTA whose
+// share lies inside one unit has none.)
 template <typename L>
 __host__ __device__ __forceinline__ int32_t first_unit(const L& a, int32_t c, int32_t grid) {
   const int64_t x = a.total_cost * c / grid;
-  int32_t j = 0;
-  while (j + 1 < a.nmats && x >= a.m[j + 1].cbeg) ++j;
+  const int32_t j = matrix_at(a.nmats, x, [&](int32_t i) { return a.m[i].cbeg; });
   return a.m[j].ubeg + static_cast<int32_t>((x - a.m[j].cbeg + a.m[j].cost - 1) / a.m[j].cost);
 }
 
@@ -74,7 +87,7 @@ struct Launch {
   int32_t oPlan, oMask;  // shared memory (bytes): plan columns, group masks; pair buffers at 0
   int64_t total_cost;    // sum over the matrices of ntiles * cost
   float* partial;        // [(grid + nmats) * stride] dC partial sums, slot = cta + matrix
-  Shape sh[kMaxShapes];
+  Shape sh[kMaxMats];    // distinct geometries
   Mat m[kMaxMats];
 };
 
@@ -538,7 +551,19 @@ __global__ void __launch_bounds__(NT, NT == 512 ? 1 : 2) fft_tile_kernel(const _
 
   const int u_begin = first_unit(args, blockIdx.x, gridDim.x);
   const int u_end = blockIdx.x + 1 == gridDim.x ? args.total_units : first_unit(args, blockIdx.x + 1, gridDim.x);
-  if (u_begin >= u_end) return;
+  if (u_begin >= u_end) {
+    // no unit: the dC reduction still sums this CTA's slot of a matrix with units
+    // on both sides of it
+    if (C && u_begin < args.total_units) {
+      const int k = matrix_at(args.nmats, u_begin, [&](int32_t i) { return args.m[i].ubeg; });
+      if (u_begin > args.m[k].ubeg) {
+        float* dst = args.partial + static_cast<size_t>(blockIdx.x + k) * args.stride;
+        const int nnz = reinterpret_cast<const FfbPlanHeader*>(args.m[k].plan)->nnz;
+        for (int q = tid; q < nnz; q += NT) dst[q] = 0.f;
+      }
+    }
+    return;
+  }
 
   // slots of frame columns in the pair buffers
   int G0 = 0, G1 = 0, cnt0 = 0, cnt1 = 0;
@@ -622,7 +647,8 @@ __global__ void __launch_bounds__(NT, NT == 512 ? 1 : 2) fft_tile_kernel(const _
   using Chunk = std::conditional_t<BIG, Big, Cols>;
   Chunk ch{};
   float dc[BIG ? 1 : KE];
-  int cur = -1, j = 0, nfZ = 0, nfix = 0, PP = 1;
+  int cur = -1, j = matrix_at(args.nmats, u_begin, [&](int32_t i) { return args.m[i].ubeg; });
+  int nfZ = 0, nfix = 0, PP = 1;
   const uint8_t* plan = nullptr;
   auto flush = [&](int mat) {
     if (!C) return;
@@ -643,7 +669,6 @@ __global__ void __launch_bounds__(NT, NT == 512 ? 1 : 2) fft_tile_kernel(const _
     }
   };
 
-  while (u_begin >= args.m[j].ubeg + args.m[j].ntiles) ++j;
   int64_t tp0 = 0;  // the previous unit (of the same matrix): first token, tokens
   int tp = 0;
   for (int u = u_begin; u < u_end; ++u) {

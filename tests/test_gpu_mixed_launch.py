@@ -1,0 +1,67 @@
+"""One launch of the group kernel over matrices of unlike cost, over plans of their
+own, and fewer units than CTAs: results against the fp64 oracle (fp32 bar), and a
+workspace that serves every smaller token count."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from paper_2608_26430_gb300 import framefb as ffb
+from paper_2608_26430_gb300 import workloads as wl
+from paper_2608_26430_gb300.batch import AdapterBatch
+from tests.oracle_side import Expect, assert_f32, host64
+
+pytestmark = pytest.mark.gpu
+
+DEV = "cuda:0"
+ALL = ffb.OP_FORWARD | ffb.OP_BACKWARD_DX | ffb.OP_GRAD_COEFF
+MIXED = [(1024, 1024)] + [(256, 256)] * 5
+UNLIKE = [(256, 256), (4096, 256), (256, 256), (256, 2048)]
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2608_26430_gb300.build import build
+    build()
+    ffb.lib()
+
+
+def load(mats, N, nnz, **kw):
+    return AdapterBatch(wl.Workload("mixed", tuple(wl.MatSpec(f"w{i}", n, m) for i, (n, m) in enumerate(mats)), N=N,
+                                    nnz=nnz, dtype="f32", c_std=0.02, **kw), DEV, ops=ALL)
+
+
+def first(b, N):
+    out = []
+    for m in b.mats:
+        c = ffb.framefb_mat.from_buffer_copy(m)
+        c.N = N
+        out.append(c)
+    return out
+
+
+@pytest.mark.parametrize("mats,nnz", [(MIXED, 1000), (UNLIKE, 500)])
+def test_one_workspace_serves_fewer_tokens(mats, nnz):
+    b = load(mats, 700, nnz)
+    sizes = [ffb.framefb_workspace_size(first(b, N), ALL) for N in range(1, 701)]
+    assert sizes == sorted(sizes)
+    for N in (150, 202, 203, 204, 405, 406, 407):
+        ws = torch.empty(sizes[N], dtype=torch.uint8, device=DEV)  # of N + 1 tokens
+        ffb.framefb_run(first(b, N), ALL, b.dtype_code, ws)
+    torch.cuda.synchronize()
+
+
+@pytest.mark.parametrize("mats,nnz,N,kw", [(MIXED, 1000, 203, {}), (UNLIKE, 500, 1, {}), (UNLIKE, 500, 64, {}),
+                                           (UNLIKE, 500, 333, {}), ([(256, 256)] * 20, 128, 9, {"per_layer_support": True}),
+                                           ([(512, 256)] * 9, 3000, 5, {"per_layer_support": True})])
+def test_parity(mats, nnz, N, kw):
+    b = load(mats, N, nnz, **kw)
+    b.run(ALL, b.workspace(ALL))
+    torch.cuda.synchronize()
+    for j, x in enumerate(b.bufs):
+        e, X, dY = Expect(b, j), host64(x.X), host64(x.dY)
+        assert_f32(host64(x.Y), e.y(X, np.zeros((N, x.spec.m))), what=f"Y[{j}]")
+        assert_f32(host64(x.dX), e.dx(dY, np.zeros((N, x.spec.n))), what=f"dX[{j}]")
+        assert_f32(host64(x.dC), e.dc(X, dY), what=f"dC[{j}]")
