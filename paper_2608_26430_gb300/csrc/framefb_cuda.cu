@@ -994,6 +994,58 @@ extern "C" framefb_status framefb_fused_fwd_bwd(const framefb_mat* mats, int32_t
                      ws_bytes, stream);
 }
 
+namespace {
+
+// CTAs of a merge: every out group's tenants in `chunks` runs and its blocks in
+// `splits` runs (a block per warp at least).
+struct MergeSplit {
+  int32_t chunks, splits;
+};
+
+// Costs in units of one block of two tenants (0.3 us of a CTA): an entry of two
+// tenants 0.08, the start of a CTA (factors, entries, values) 8.  A merge of more
+// than 100 units per resident CTA goes in some eight waves of CTAs of four pairs of
+// tenants, the out group with most entries (`most`) in parts of at most two CTAs'
+// work (64 tenants, bf16, against one wave of equal parts: 4096^2 653 -> 363 us, with
+// Zipf rows 1483 -> 365; 768 -> 3072 75 -> 61); a smaller one, or one pair of tenants,
+// takes the split with the least estimated time, waves of average CTAs and then one
+// of that out group (one tenant of 4096^2, Zipf rows, 22 -> 18; of 4096 -> 14336,
+// 448 out groups, 60 -> 46).
+MergeSplit merge_split(int32_t Gm, int32_t Gn, int32_t nnz, int32_t most, int32_t T, int64_t resident) {
+  constexpr double kEntry = 0.08, kStart = 8.0;
+  const int64_t pairs = (static_cast<int64_t>(T) + 1) / 2, most_splits = (Gn + ffb::kMergeWarps - 1) / ffb::kMergeWarps;
+  const double mean = static_cast<double>(nnz) / Gm;
+  const double work = static_cast<double>(pairs) * Gm * (Gn + kEntry * mean) / static_cast<double>(resident);
+  if (pairs > 1 && work > 100) {
+    const double aim = std::max(24.0, work / 8);
+    const int64_t per = std::min<int64_t>(pairs, 4);
+    const double splits = std::max(per * (Gn + kEntry * mean) / aim, per * (Gn + kEntry * most) / (2 * aim));
+    return MergeSplit{static_cast<int32_t>((pairs + per - 1) / per),
+                      static_cast<int32_t>(std::min<int64_t>(most_splits, std::max<int64_t>(1, std::llround(splits))))};
+  }
+  MergeSplit best{1, 1};
+  double least = 1e300;
+  int64_t last = 0;
+  // few large CTAs first: smaller ones have to be clearly better
+  for (int64_t per = pairs; per > 0; per = per <= 4 ? per - 1 : per - per / 3) {  // pairs of tenants per CTA
+    const int64_t chunks = (pairs + per - 1) / per;
+    if (chunks == last) continue;
+    last = chunks;
+    for (int64_t splits = 1; splits <= most_splits; splits += splits < 4 ? 1 : splits / 2) {
+      const double blocks = static_cast<double>((Gn + splits - 1) / splits);
+      const double avg = per * (blocks + kEntry * mean / splits) + kStart, top = per * (blocks + kEntry * most / splits) + kStart;
+      const double t = static_cast<double>((Gm * chunks * splits - 1) / resident) * avg + top;
+      if (t < 0.95 * least) {
+        least = t;
+        best = MergeSplit{static_cast<int32_t>(chunks), static_cast<int32_t>(splits)};
+      }
+    }
+  }
+  return best;
+}
+
+}  // namespace
+
 extern "C" framefb_status framefb_merge(const void* W0, framefb_dtype dtype, int32_t m, int32_t n, int64_t ldw,
                                         const framefb_dev_frame* fin, const framefb_dev_frame* fout,
                                         const framefb_plan* plan, const void* plan_dev, const float* c_vals,
@@ -1036,20 +1088,17 @@ extern "C" framefb_status framefb_merge(const void* W0, framefb_dtype dtype, int
   if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, ffb::kMergeThreads, 0) != cudaSuccess)
     return FRAMEFB_ECUDA;
-  // one wave of CTAs: the tenants of an out group in as many runs as are
-  // resident, then (few tenants) its blocks in runs of at least a warp each
-  const int64_t resident = std::max<int64_t>(1, static_cast<int64_t>(sms) * std::max(per_sm, 1));
-  // (tenants go in twos: an odd run would end on a half-used pass)
-  const int64_t chunks = std::max<int64_t>(1, std::min<int64_t>((T + 1) / 2, resident / h->Gm));
-  const int64_t splits = std::max<int64_t>(
-      1, std::min<int64_t>((h->Gn + ffb::kMergeWarps - 1) / ffb::kMergeWarps, resident / (h->Gm * chunks)));
+  const MergeSplit sp = merge_split(h->Gm, h->Gn, h->nnz, plan->merge_most, T, static_cast<int64_t>(sms) * std::max(per_sm, 1));
   a.Gn = h->Gn;
   a.Gm = h->Gm;
   a.off_blkptr = h->off_blkptr;
   a.off_blkent = h->off_blkent;
-  a.chunks = static_cast<int32_t>(chunks);
-  a.splits = static_cast<int32_t>(splits);
-  const int64_t grid = static_cast<int64_t>(h->Gm) * chunks * splits;
+  a.chunks = sp.chunks;
+  a.splits = sp.splits;
+  // bf16 and W0 of more than half of L2 (4096^2, one tenant, with W0 in L2: 11.6 us without, 13.1 with;
+  // fp32 rows are whole lines and gain nothing)
+  a.ahead = esz == 2 && static_cast<size_t>(m) * ldw * esz > (size_t{64} << 20);
+  const int64_t grid = static_cast<int64_t>(h->Gm) * sp.chunks * sp.splits;
   if (ffb_host::launch_chained(fn, dim3(static_cast<unsigned>(grid)), dim3(ffb::kMergeThreads), kargs, 0,
                        static_cast<cudaStream_t>(stream)) != cudaSuccess)
     return FRAMEFB_ECUDA;

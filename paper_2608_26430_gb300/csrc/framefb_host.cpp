@@ -901,6 +901,8 @@ extern "C" framefb_status framefb_plan_build(const framefb_frame* fin, const fra
     framefb_plan* plan = new framefb_plan;
     std::unique_ptr<framefb_plan> guard(plan);
     plan->image = std::move(image);
+    std::vector<int32_t> per_group(Gm, 0);
+    for (const Entry& e : ent) plan->merge_most = std::max(plan->merge_most, ++per_group[e.key0 / FFB_GROUP]);
     if (parts) {
       const std::vector<Block> bo = side_blocks(Gm), bi = side_blocks(Gn);
       // the parts' entries first; their plans are built side by side

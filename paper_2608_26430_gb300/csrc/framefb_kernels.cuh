@@ -91,6 +91,7 @@ struct MergeK {
   int64_t ldw;
   int32_t m, n, rho_in, rho_out, nnz, T;
   int32_t splits, chunks;  // CTAs per out group: runs of blocks x runs of tenants
+  int32_t ahead;           // W0 comes from DRAM in half lines: ask for the next block early
   int32_t Gn, Gm, off_blkptr, off_blkent;  // of the plan
   float seff;
 };
@@ -761,19 +762,21 @@ __global__ void __launch_bounds__(256) dc_reduce_kernel(const __grid_constant__ 
 // Merge (Sec. 3.4 "Storage efficiency", Alg. 1 step 6 per tenant):
 //   W_t[32g + i][32h + j] = W0[..] + (s/16) sum_{e in block (g,h)} c_{t,e} Dout[i][a_e] Din[j][b_e],
 // D = 4 x the group-0 block of each frame (k = 16, k*rho = d frames).  A CTA
-// takes one out group g, a run of its 32 x 32 blocks h and a run of tenants: the
-// entries of the blocks (contiguous in the plan) and the tenants' values of them
-// are staged in shared memory once, so no global load sits in the loops.  A warp
+// takes one out group g, a run of its 32 x 32 blocks h and a run of tenants
+// (framefb_cuda.cu, merge_split): the entries of the blocks (contiguous in the
+// plan) and the tenants' values of them are staged in shared memory, as many
+// blocks at a time as fit, so no global load sits in the entry loop.  A warp
 // takes blocks in turn and two tenants at a time: W0, the frame factors and the
 // entries are read once for both, and the products run on pairs of columns
 // (fp32x2).  A lane owns one 16-byte chunk of one row per row pass: lanes (row
 // l / CPR, chunk l % CPR), CPR = 16-byte chunks per 32-element row (4 bf16, 8
-// fp32), so a warp's store covers whole 64- or 128-byte row segments.  Bound:
-// the writes of W_t: 64 tenants of 768^2, 2000 entries, take 26.4 us in bf16
-// (75 MB) and 33 us in fp32, 19 us of the former without any entry; 8 tenants of
-// 4096^2 59 us (5.1 TB/s).  With one warp per (group, tenant, four blocks) that
-// staged its own entries the loads' latency and the factors' re-reads bounded
-// it: 30, 39.5 and 77 us.
+// fp32), so a warp's store covers whole 64- or 128-byte row segments.  Bound: the
+// writes of W_t (64 tenants of 4096^2 in bf16 363 us, 5.9 TB/s; 8 of 8192^2 in fp32
+// 400 us, 5.4 TB/s); 64 of 768^2, 2000 entries, 22.6 us (75 MB, 19 us without any
+// entry) in bf16 and 31 us in fp32: waves of few blocks.  With one warp per (group,
+// tenant, four blocks) that staged its own entries the loads' latency and the
+// factors' re-reads bounded it: 603, 664, 30 and 39 us (one tenant of 8192^2 in fp32,
+// all reads and writes of DRAM, 89 us there and 102 here).
 // ---------------------------------------------------------------------------
 template <typename Elem>
 struct MergeIO;
@@ -814,7 +817,7 @@ struct MergeIO<float> {
 
 constexpr int kMergeThreads = 256;
 constexpr int kMergeWarps = kMergeThreads / 32;
-constexpr int kMergeEnt = 1024;  // entries a CTA stages (longer runs of blocks read them from L2)
+constexpr int kMergeEnt = 2048;  // entries a CTA stages at a time (a block has at most 1024)
 constexpr int kMergeBlk = 1024;  // blocks of an out group (a plan has at most 32768 columns)
 constexpr int kMergeVal = 4096;  // staged coefficient values: tenants x entries
 
@@ -846,31 +849,21 @@ __global__ void __launch_bounds__(kMergeThreads, 2) merge_kernel(const __grid_co
   __shared__ float2 Dout2[32][33];              // [a][i] = (Dout[i][a], Dout[i][a])
   __shared__ __align__(16) float DinT[32][32];  // [b][j] = Din[j][b]
   __shared__ int32_t ent_s[kMergeEnt];          // a_local | b_local << 8
-  __shared__ int32_t q_s[kMergeEnt];            // index of its value
-  __shared__ float cv_s[kMergeVal];             // [tenant][entry]
-  __shared__ int32_t ptr_s[kMergeBlk + 1];      // entry ranges of the CTA's blocks (from its first entry)
+  __shared__ __align__(8) float cv_s[kMergeVal];  // [pair of tenants][entry][tenant of the pair]
+  __shared__ int32_t ptr_s[kMergeBlk + 1];      // entry ranges of the CTA's blocks
   const int2* blkent = table<int2>(a.plan, a.off_blkent);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int rl = lane / CPR, cl = lane % CPR;  // row in the pass, chunk in the row
   // this CTA's out group, blocks [h0, h1) and tenants [t0, t1)
-  const int g = blockIdx.x % a.Gm, part = blockIdx.x / a.Gm;
+  const int parts = a.splits * a.chunks, g = blockIdx.x / parts, part = blockIdx.x - g * parts;
   const int split = part % a.splits, chunk = part / a.splits;
   const int h0 = static_cast<int>(static_cast<int64_t>(a.Gn) * split / a.splits);
   const int h1 = static_cast<int>(static_cast<int64_t>(a.Gn) * (split + 1) / a.splits);
   const int64_t pairs = (static_cast<int64_t>(a.T) + 1) / 2;  // tenants go in twos
-  const int64_t t0 = 2 * (pairs * chunk / a.chunks), t1 = min(static_cast<int64_t>(a.T), 2 * (pairs * (chunk + 1) / a.chunks));
+  const int t0 = static_cast<int>(2 * (pairs * chunk / a.chunks));
+  const int t1 = static_cast<int>(min(static_cast<int64_t>(a.T), 2 * (pairs * (chunk + 1) / a.chunks)));
   const int32_t* blkptr = table<int32_t>(a.plan, a.off_blkptr) + g * a.Gn + h0;
-  const int eg0 = ld_g(blkptr), ne = ld_g(blkptr + (h1 - h0)) - eg0;
-  for (int x = threadIdx.x; x <= h1 - h0; x += kMergeThreads) ptr_s[x] = ld_g(blkptr + x) - eg0;
-  const bool staged = ne <= kMergeEnt;
-  const int tb = staged ? (ne > 0 ? min(static_cast<int64_t>(kMergeVal / ne), t1 - t0) : t1 - t0) : t1 - t0;  // tenants per batch
-  if (staged) {
-    for (int e = threadIdx.x; e < ne; e += kMergeThreads) {
-      const int2 en = ld_g(blkent + eg0 + e);
-      ent_s[e] = en.x;
-      q_s[e] = en.y;
-    }
-  }
+  for (int x = threadIdx.x; x <= h1 - h0; x += kMergeThreads) ptr_s[x] = ld_g(blkptr + x);
   for (int idx = threadIdx.x; idx < 1024; idx += kMergeThreads) {
     const int w = idx & 31, x = idx >> 5, i = x >> 1, s = x & 1;  // column x = 2i + s of the group block, row w
     const float o = 4.f * ld_g(a.fout_val + 32 * (i * a.rho_out + s) + w);
@@ -880,91 +873,104 @@ __global__ void __launch_bounds__(kMergeThreads, 2) merge_kernel(const __grid_co
   const Elem* W0 = static_cast<const Elem*>(a.W0) + static_cast<int64_t>(32 * g + rl) * a.ldw + cl * PER;
   const int64_t tstride = static_cast<int64_t>(a.m) * a.ldw;
   const uint64_t seff2 = f2_pack(a.seff, a.seff);
-  for (int64_t tb0 = t0; tb0 < t1; tb0 += tb) {
-    const int nt = static_cast<int>(min(static_cast<int64_t>(tb), t1 - tb0));
-    __syncthreads();  // entries staged; the previous batch's values are no longer read
-    if (staged) {
+  __syncthreads();
+  // runs of blocks [ha, hr) whose entries fit the stage, and tenants of a run whose
+  // values do
+  for (int ha = h0, hr; ha < h1; ha = hr) {
+    const int eg0 = ptr_s[ha - h0];
+    hr = h1;
+    if (ptr_s[h1 - h0] - eg0 > kMergeEnt) {
+      int lo = ha + 1, hi = h1 - 1;
+      while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (ptr_s[mid - h0] - eg0 <= kMergeEnt)
+          lo = mid;
+        else
+          hi = mid - 1;
+      }
+      hr = lo;
+    }
+    const int ne = ptr_s[hr - h0] - eg0;
+    const int tb = ne > 0 ? min(kMergeVal / ne & ~1, t1 - t0) : t1 - t0;  // (even, or the last)
+    for (int tb0 = t0; tb0 < t1; tb0 += tb) {
+      const int nt = min(tb, t1 - tb0);
+      if (ha > h0 || tb0 > t0) __syncthreads();  // the previous entries and values are no longer read
+      if (tb0 == t0)
+        for (int e = threadIdx.x; e < ne; e += kMergeThreads) ent_s[e] = ld_g(&blkent[eg0 + e].x);
       for (int x = threadIdx.x; x < nt * ne; x += kMergeThreads) {
         const int t = x / ne, e = x - t * ne;
-        cv_s[x] = ld_g(a.c_vals + (tb0 + t) * a.nnz + q_s[e]);
+        cv_s[2 * ((t >> 1) * ne + e) + (t & 1)] = ld_g(a.c_vals + static_cast<int64_t>(tb0 + t) * a.nnz + ld_g(&blkent[eg0 + e].y));
       }
-    }
-    __syncthreads();
-    for (int hb = h0 + warp; hb < h1; hb += kMergeWarps) {
-      const int e0 = ptr_s[hb - h0], e1 = ptr_s[hb - h0 + 1];
-      uint64_t w0[PASSES][PER / 2];
+      __syncthreads();
+      for (int hb = ha + warp; hb < hr; hb += kMergeWarps) {
+        const int e0 = ptr_s[hb - h0] - eg0, e1 = ptr_s[hb - h0 + 1] - eg0;
+        // the warp's next block of W0 towards L2, a row per lane (one tenant of
+        // 14336 -> 4096 in bf16 without: 53.5 us, with 43.2)
+        if (a.ahead && hb + kMergeWarps < h1)
+          asm volatile("prefetch.global.L2 [%0];" ::"l"(static_cast<const Elem*>(a.W0) + static_cast<int64_t>(32 * g + lane) * a.ldw +
+                                                        32 * (hb + kMergeWarps)));
+        uint4 w0[PASSES];
 #pragma unroll
-      for (int r = 0; r < PASSES; ++r) {
-        float w[PER];
-        IO::unpack(ld_g(reinterpret_cast<const uint4*>(W0 + static_cast<int64_t>(r * RPP) * a.ldw + 32 * hb)), w);
+        for (int r = 0; r < PASSES; ++r)
+          w0[r] = ld_g(reinterpret_cast<const uint4*>(W0 + static_cast<int64_t>(r * RPP) * a.ldw + 32 * hb));
+        // TT tenants from batch tenant t on
+        auto tenants = [&](auto tt, int t) {
+          constexpr int TT = decltype(tt)::value;
+          uint64_t acc[TT][PASSES][PER / 2];
 #pragma unroll
-        for (int j = 0; j < PER / 2; ++j) w0[r][j] = f2_pack(w[2 * j], w[2 * j + 1]);
-      }
-      // TT tenants from batch tenant t on
-      auto tenants = [&](auto tt, int t) {
-        constexpr int TT = decltype(tt)::value;
-        uint64_t acc[TT][PASSES][PER / 2];
+          for (int k = 0; k < TT; ++k)
 #pragma unroll
-        for (int k = 0; k < TT; ++k)
+            for (int r = 0; r < PASSES; ++r)
 #pragma unroll
-          for (int r = 0; r < PASSES; ++r)
+              for (int j = 0; j < PER / 2; ++j) acc[k][r][j] = 0ull;
+          for (int e = e0; e < e1; ++e) {
+            const int ex = ent_s[e];
+            const float2 cp = reinterpret_cast<const float2*>(cv_s)[(t >> 1) * ne + e];
+            const float c[2] = {cp.x, cp.y};
+            const int al = ex & 31, bl = (ex >> 8) & 31;
+            uint64_t din[PER / 2];
 #pragma unroll
-            for (int j = 0; j < PER / 2; ++j) acc[k][r][j] = 0ull;
-        for (int e = e0; e < e1; ++e) {
-          int ex;
-          float c[TT];
-          if (staged) {
-            ex = ent_s[e];
+            for (int j = 0; j < PER / 2; j += 2) {
+              const ulonglong2 q = *reinterpret_cast<const ulonglong2*>(&DinT[bl][cl * PER + 2 * j]);
+              din[j] = q.x;
+              din[j + 1] = q.y;
+            }
+            uint64_t u[PASSES];
 #pragma unroll
-            for (int k = 0; k < TT; ++k) c[k] = cv_s[(t + k) * ne + e];
-          } else {
-            const int2 en = ld_g(blkent + eg0 + e);
-            ex = en.x;
+            for (int r = 0; r < PASSES; ++r) u[r] = *reinterpret_cast<const uint64_t*>(&Dout2[al][r * RPP + rl]);
 #pragma unroll
-            for (int k = 0; k < TT; ++k) c[k] = ld_g(a.c_vals + (tb0 + t + k) * a.nnz + en.y);
+            for (int k = 0; k < TT; ++k) {
+              const uint64_t cc = f2_pack(c[k], c[k]);
+#pragma unroll
+              for (int j = 0; j < PER / 2; ++j) {
+                const uint64_t cd = f2_mul(cc, din[j]);
+#pragma unroll
+                for (int r = 0; r < PASSES; ++r) acc[k][r][j] = f2_fma(u[r], cd, acc[k][r][j]);
+              }
+            }
           }
-          const int al = ex & 31, bl = (ex >> 8) & 31;
-          uint64_t din[PER / 2];
-#pragma unroll
-          for (int j = 0; j < PER / 2; j += 2) {
-            const ulonglong2 q = *reinterpret_cast<const ulonglong2*>(&DinT[bl][cl * PER + 2 * j]);
-            din[j] = q.x;
-            din[j + 1] = q.y;
-          }
-          uint64_t u[PASSES];
-#pragma unroll
-          for (int r = 0; r < PASSES; ++r) u[r] = *reinterpret_cast<const uint64_t*>(&Dout2[al][r * RPP + rl]);
 #pragma unroll
           for (int k = 0; k < TT; ++k) {
-            const uint64_t cc = f2_pack(c[k], c[k]);
+            Elem* Wt = static_cast<Elem*>(a.Wout) + (tb0 + t + k) * tstride + static_cast<int64_t>(32 * g + rl) * a.ldw +
+                      cl * PER + 32 * hb;
 #pragma unroll
-            for (int j = 0; j < PER / 2; ++j) {
-              const uint64_t cd = f2_mul(cc, din[j]);
+            for (int r = 0; r < PASSES; ++r) {
+              float w[PER];
+              IO::unpack(w0[r], w);
 #pragma unroll
-              for (int r = 0; r < PASSES; ++r) acc[k][r][j] = f2_fma(u[r], cd, acc[k][r][j]);
+              for (int j = 0; j < PER / 2; ++j) {
+                const uint64_t x = f2_fma(seff2, acc[k][r][j], f2_pack(w[2 * j], w[2 * j + 1]));
+                asm("mov.b64 {%0, %1}, %2;" : "=f"(w[2 * j]), "=f"(w[2 * j + 1]) : "l"(x));
+              }
+              // (written once, not read here: streaming stores leave L2 sooner, fp32 39 -> 33 us)
+              __stcs(reinterpret_cast<uint4*>(Wt + static_cast<int64_t>(r * RPP) * a.ldw), IO::pack(w));
             }
           }
-        }
-#pragma unroll
-        for (int k = 0; k < TT; ++k) {
-          Elem* Wt = static_cast<Elem*>(a.Wout) + (tb0 + t + k) * tstride + static_cast<int64_t>(32 * g + rl) * a.ldw +
-                     cl * PER + 32 * hb;
-#pragma unroll
-          for (int r = 0; r < PASSES; ++r) {
-            float w[PER];
-#pragma unroll
-            for (int j = 0; j < PER / 2; ++j) {
-              const uint64_t x = f2_fma(seff2, acc[k][r][j], w0[r][j]);
-              asm("mov.b64 {%0, %1}, %2;" : "=f"(w[2 * j]), "=f"(w[2 * j + 1]) : "l"(x));
-            }
-            // (written once, not read here: streaming stores leave L2 sooner, fp32 39 -> 33 us)
-            __stcs(reinterpret_cast<uint4*>(Wt + static_cast<int64_t>(r * RPP) * a.ldw), IO::pack(w));
-          }
-        }
-      };
-      int t = 0;
-      for (; t + 2 <= nt; t += 2) tenants(std::integral_constant<int, 2>{}, t);
-      if (t < nt) tenants(std::integral_constant<int, 1>{}, t);
+        };
+        int t = 0;
+        for (; t + 2 <= nt; t += 2) tenants(std::integral_constant<int, 2>{}, t);
+        if (t < nt) tenants(std::integral_constant<int, 1>{}, t);
+      }
     }
   }
 }

@@ -20,6 +20,7 @@ struct FfbSubPlan {
 struct framefb_plan {
   std::vector<uint8_t> image;  // device image: FfbPlanHeader and its tables, then the parts
   std::vector<FfbSubPlan> subs;
+  int32_t merge_most = 0;      // entries of the out group that holds most (merge)
   framefb_plan() = default;
   framefb_plan(const framefb_plan&) = delete;
   framefb_plan& operator=(const framefb_plan&) = delete;
