@@ -130,7 +130,7 @@ struct Prepared {
   fp::Reduce* red;
   int grid, nnz_max;
   Variant v;
-  size_t smem, ws_bytes;
+  size_t smem, ws_bytes, ws_cover;  // (workspace this launch takes, and what a query reports)
 };
 
 // One launch: as many matrices as the parameters hold, of one variant.
@@ -184,10 +184,13 @@ framefb_status prepare(const Chunk& ch, int32_t ops, framefb_dtype dt, Prepared&
     return FRAMEFB_ECUDA;
   const int per = ch.v.nt == 512 ? 1 : 2;
   const int nm = static_cast<int>(ch.mats.size());
-  // pairs per unit: what fits, but no more than gives every CTA a unit
+  // pairs per unit: what fits, but no more than one unit per CTA takes.  (Rounded
+  // up: with units of one pair and up to two per CTA, some CTAs walked two units one
+  // after the other: 256^2 fp32, 3000 entries, 512 tokens, forward 15.7 us, 11.9 so.)
+  const int64_t slots = static_cast<int64_t>(sms) * per;
   int64_t pairs = 0;
   for (const framefb_mat* M : ch.mats) pairs += (M->N + 1) / 2;
-  const int64_t spread = std::max<int64_t>(1, pairs / (static_cast<int64_t>(sms) * per));
+  const int64_t spread = std::max<int64_t>(1, (pairs + slots - 1) / slots);
   int nsh = 0;
   Regions reg;
   for (int j = 0; j < nm; ++j) {
@@ -235,13 +238,18 @@ framefb_status prepare(const Chunk& ch, int32_t ops, framefb_dtype dt, Prepared&
     K.ubeg = static_cast<int32_t>(units);
     K.ntiles = (M.N + 2 * sh.PP - 1) / (2 * sh.PP);
     K.seff = static_cast<float>(static_cast<double>(M.scale) / 16.0);
-    // a unit's cost: groups to transform and entries to gather, per pair
-    K.cost = sh.PP * (2 * (h.Gn + h.Gm) * kGroupCost + h.nnz * kEntryCost) / 64 + 1;
-    K.cbeg = A.total_cost;
-    A.total_cost += static_cast<int64_t>(K.cost) * K.ntiles;
     units += K.ntiles;
     if (units > INT32_MAX / 2) return FRAMEFB_EUNSUPPORTED;
     nnz_max = std::max(nnz_max, h.nnz);
+  }
+  // The units are split over the CTAs at equal cost: groups to transform and
+  // entries to gather, per pair; one unit per CTA where there are no more of them.
+  for (int j = 0; j < nm; ++j) {
+    const FfbPlanHeader& h = *header_of(ch.mats[j]->plan);
+    fg::Mat& K = A.m[j];
+    K.cost = units <= slots ? 1 : A.sh[K.shape].PP * (2 * (h.Gn + h.Gm) * kGroupCost + h.nnz * kEntryCost) / 64 + 1;
+    K.cbeg = A.total_cost;
+    A.total_cost += static_cast<int64_t>(K.cost) * K.ntiles;
   }
   A.nmats = nm;
   A.mode = ops;
@@ -253,28 +261,29 @@ framefb_status prepare(const Chunk& ch, int32_t ops, framefb_dtype dt, Prepared&
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, ch.v.nt, P.smem) != cudaSuccess)
     return FRAMEFB_ECUDA;
   if (per_sm < 1) return FRAMEFB_EUNSUPPORTED;
-  // As many CTAs as there are units, or as are resident.  (With a unit for every
-  // CTA at equal shares, the largest unit's cost bounded the grid: one matrix of
-  // 4096 -> 256 beside two small ones, 64 tokens, forward, then ran on 57 CTAs in
-  // 24.6 us, and the grid fell where more tokens made the units larger.)
-  P.grid = static_cast<int>(std::min<int64_t>(static_cast<int64_t>(sms) * per_sm, units));
-  P.ws_bytes = 0;
+  // (With a unit for every CTA at equal shares the largest unit's cost bounded the
+  // grid: 4096 -> 256 beside two small ones, 128 tokens, forward, 24.5 us, 10.6 so.)
+  P.grid = static_cast<int>(std::min<int64_t>({slots, static_cast<int64_t>(sms) * per_sm, units}));
+  P.ws_bytes = P.ws_cover = 0;
   if (ops & FRAMEFB_OP_GRAD_COEFF) {
-    P.ws_bytes = static_cast<size_t>(P.grid + nm) * A.stride * sizeof(float) + 256;
+    // (more tokens can make fewer, larger units: what is asked for covers the
+    // grid of any smaller count)
+    auto bytes = [&](int64_t ctas) { return static_cast<size_t>(ctas + nm) * A.stride * sizeof(float) + 256; };
+    P.ws_bytes = bytes(P.grid);
+    P.ws_cover = bytes(std::min(slots, pairs));
     P.red->stride = A.stride;
-    // CTA of unit u: the last one whose first unit is not past it
-    int32_t c = 0;
-    auto cta_of = [&](int32_t u) {
-      while (c + 1 < P.grid && fg::first_unit(A, c + 1, P.grid) <= u) ++c;
-      return c;
+    // CTA of a unit: the last one whose share begins at or before the unit
+    auto cta_of = [&](const fg::Mat& K, int32_t u) {
+      const int64_t at = K.cbeg + static_cast<int64_t>(u - K.ubeg) * K.cost;
+      return static_cast<int32_t>(((at + 1) * P.grid + A.total_cost - 1) / A.total_cost - 1);
     };
     for (int j = 0; j < nm; ++j) {
       fp::ReduceMat& R = P.red->m[j];
       R.dC = ch.mats[j]->dC;
       R.nnz = header_of(ch.mats[j]->plan)->nnz;
       R.seff = A.m[j].seff;
-      R.c0 = cta_of(A.m[j].ubeg);
-      R.c1 = cta_of(A.m[j].ubeg + A.m[j].ntiles - 1);
+      R.c0 = cta_of(A.m[j], A.m[j].ubeg);
+      R.c1 = cta_of(A.m[j], A.m[j].ubeg + A.m[j].ntiles - 1);
     }
   }
   return FRAMEFB_OK;
@@ -378,7 +387,7 @@ framefb_status grp_check(const framefb_mat* mats, int32_t nmats, int32_t ops, fr
       l.P = l.b.prep();
       const framefb_status s = prepare(c, ops, dt, l.P);
       if (s != FRAMEFB_OK) return s;
-      *ws_need = std::max(*ws_need, l.P.ws_bytes);
+      *ws_need = std::max(*ws_need, keep ? l.P.ws_bytes : l.P.ws_cover);
       l.fn = kernel_ptr(l.P.v, dt);
       l.mats = static_cast<unsigned>(c.mats.size());
       l.reduce = (ops & FRAMEFB_OP_GRAD_COEFF) && l.P.nnz_max > 0;
