@@ -750,14 +750,14 @@ bool parts_allowed() {
 //     22 / 44 / 106 against 19 / 35 / 95; with dX the parts take turns, fused pass
 //     32 / 71 / 188 against 91 / 140 / 300.
 // (FRAMEFB_PARTS=0 leaves the other bf16 plans to the contraction path.)
-bool group_route(const framefb_mat& M, const FfbPlanHeader& h, int32_t ops, framefb_dtype dt) {
+bool group_route(const framefb_mat& M, const FfbPlanHeader& h, ffb_host::GrpKind kind, int32_t ops, framefb_dtype dt) {
   if (!tc_allowed()) return false;
   if (dt == FRAMEFB_BF16) {
     if (fused_tc_ok(h) || !parts_allowed()) return false;
     const bool short_columns = h.EZ <= ffb::kEreg && h.EG <= ffb::kEreg;
     if (!(ops & FRAMEFB_OP_BACKWARD_DX) && short_columns && !M.plan->subs.empty()) return false;
   }
-  return ffb_host::grp_takes(M, ops, dt);
+  return ffb_host::grp_takes(kind, M, ops, dt);
 }
 
 // Matrices of a call split by path, each in call order: the row-transform
@@ -775,16 +775,18 @@ framefb_status split_paths(const framefb_mat* mats, int32_t nmats, int32_t ops, 
                            std::vector<framefb_mat>& grp, std::vector<framefb_mat>& den, std::vector<framefb_mat>& row,
                            std::vector<framefb_mat>& fft,
                            std::vector<framefb_mat>* prt = nullptr) {
+  ffb_host::GrpKind kind = ffb_host::GrpKind::none;
   try {
     for (int32_t j = 0; j < nmats; ++j) {
       const framefb_mat& M = mats[j];
       const FfbPlanHeader* h = plan_header(M.plan);
       if (!h) return FRAMEFB_EINVAL;
+      if (j == 0 || M.plan != mats[j - 1].plan) kind = ffb_host::grp_kind(M.plan);  // (matrices of one plan come in runs)
       if (ffb_host::row_takes(M, ops, dt)) {
         row.push_back(M);
         continue;
       }
-      if (group_route(M, *h, ops, dt)) {
+      if (group_route(M, *h, kind, ops, dt)) {
         fft.push_back(M);
         continue;
       }

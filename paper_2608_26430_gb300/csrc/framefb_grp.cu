@@ -130,7 +130,8 @@ struct Prepared {
   fp::Reduce* red;
   int grid, nnz_max;
   Variant v;
-  size_t smem, ws_bytes, ws_cover;  // (workspace this launch takes, and what a query reports)
+  int64_t slots;  // CTAs that are resident
+  size_t smem, ws_bytes;
 };
 
 // One launch: as many matrices as the parameters hold, of one variant.
@@ -264,13 +265,10 @@ framefb_status prepare(const Chunk& ch, int32_t ops, framefb_dtype dt, Prepared&
   // (With a unit for every CTA at equal shares the largest unit's cost bounded the
   // grid: 4096 -> 256 beside two small ones, 128 tokens, forward, 24.5 us, 10.6 so.)
   P.grid = static_cast<int>(std::min<int64_t>({slots, static_cast<int64_t>(sms) * per_sm, units}));
-  P.ws_bytes = P.ws_cover = 0;
+  P.slots = slots;
+  P.ws_bytes = 0;
   if (ops & FRAMEFB_OP_GRAD_COEFF) {
-    // (more tokens can make fewer, larger units: what is asked for covers the
-    // grid of any smaller count)
-    auto bytes = [&](int64_t ctas) { return static_cast<size_t>(ctas + nm) * A.stride * sizeof(float) + 256; };
-    P.ws_bytes = bytes(P.grid);
-    P.ws_cover = bytes(std::min(slots, pairs));
+    P.ws_bytes = static_cast<size_t>(P.grid + nm) * A.stride * sizeof(float) + 256;
     P.red->stride = A.stride;
     // CTA of a unit: the last one whose share begins at or before the unit
     auto cta_of = [&](const fg::Mat& K, int32_t u) {
@@ -329,27 +327,49 @@ framefb_status check_mat(const framefb_mat& M, int32_t ops, framefb_dtype dt) {
 }  // namespace
 
 // The path takes
-//   * fp32: every structured plan that fits a variant (the one-phase FFT kernel
-//     keeps the others).  Fused pass, that kernel -> this one: 8 matrices of
-//     768^2, 2048 tokens 203 -> 107 us; 2 of 3072^2, 1000 tokens 85 -> 63 us; 8 of
-//     256^2, 4096 tokens 277 -> 90 us; 8 tokens of one of 256^2 the same 21 us.
+//   * fp32: every structured plan that fits a variant with whole buffers.  Fused
+//     pass, the one-phase FFT kernel -> this one: 8 matrices of 768^2, 2048 tokens
+//     203 -> 104 us; 4096^2, 1000 entries, 256 tokens 34 -> 22; 96 of 256^2, 512
+//     tokens 440 -> 123; 8 tokens of one of 256^2 the same 13 us.
+//   * fp32 with compacted buffers (BIG), where it is the faster one.  Columns of up
+//     to 16 entries come here for their wide sides only (8192, 14336 features), and
+//     the transforms of mostly unnamed coordinates gain nothing: 14336 -> 4096, 1000
+//     entries, fused, 8 / 256 / 2000 tokens 24 / 42 / 185 us there, 32 / 35 / 196
+//     here.  Longer columns: passes with dX and dC (4096^2, 8192 entries, 8 / 1024
+//     tokens 64 / 173 -> 54 / 99; 4096 -> 14336 57 / 335 -> 52 / 153; an input side
+//     of more than 256 groups from 160 tokens, 14336 -> 4096 at 128 / 202 tokens 62 /
+//     109 against 69 / 70); a forward pass on 8192 features and more of both sides
+//     (4096^2 31 / 57 -> 21 / 41, but 4096 -> 1024, 1024 tokens 35 -> 41); dX or dC
+//     alone there from 768 tokens (4096^2, 512 / 1024 / 2000 tokens, dX 31 / 56 / 107
+//     against 36 / 48 / 66).
 //   * bf16: plans beyond the tcgen05 kernels with a side of more than 128
 //     groups (the LLaMA-3 MLP shapes), whole: the tcgen05 kernel would run them
 //     in parts or not at all.  8192 Zipf entries, fused, 64 / 1024 / 4096 tokens:
-//     4096 -> 14336 (five parts) 115 / 194 / 408 -> 49 / 102 / 249 us;
-//     14336 -> 4096 (contraction path) 61 / 220 / 664 -> 61 / 112 / 268 us, so
+//     4096 -> 14336 (five parts) 112 / 193 / 412 -> 43 / 99 / 248 us, 4096 -> 5120
+//     74 / 125 / 263 -> 38 / 74 / 199;
+//     14336 -> 4096 (contraction path) 61 / 218 / 660 -> 61 / 109 / 265 us, so
 //     that side from 128 tokens.  Narrower big plans stay in parts (4096^2, 8192
 //     tokens 289 us against 340 here).
 constexpr int32_t kMinTokensWideIn = 128;
+constexpr int32_t kBigGroups = 256;      // of both sides: a forward pass, dX or dC alone
+constexpr int32_t kBigTokensWideIn = 160, kBigTokensOne = 768;
 
-bool grp_takes(const framefb_mat& M, int32_t ops, framefb_dtype dt) {
-  (void)ops;
+GrpKind grp_kind(const framefb_plan* plan) {
+  const FfbPlanHeader* h = header_of(plan);
+  const Variant v = h ? variant(h) : Variant{0, 0, false};
+  return v.nt == 0 ? GrpKind::none : v.big ? GrpKind::big : GrpKind::whole;
+}
+
+bool grp_takes(GrpKind kind, const framefb_mat& M, int32_t ops, framefb_dtype dt) {
+  if (kind == GrpKind::none || M.N < 1) return false;
+  if (kind == GrpKind::whole) return dt == FRAMEFB_F32;
   const FfbPlanHeader* h = header_of(M.plan);
-  if (!h || M.N < 1) return false;
-  const Variant v = variant(h);
-  if (v.nt == 0) return false;
-  if (dt == FRAMEFB_F32) return true;
-  return v.big && (h->Gm > 128 || (h->Gn > 128 && M.N >= kMinTokensWideIn));
+  if (dt == FRAMEFB_BF16) return h->Gm > 128 || (h->Gn > 128 && M.N >= kMinTokensWideIn);
+  const bool D = ops & FRAMEFB_OP_BACKWARD_DX, C = ops & FRAMEFB_OP_GRAD_COEFF;
+  if (static_cast<size_t>(ffb_tile_layout(*h, ops, 1, C).total) * 4 > 227 * 1024) return true;  // too large for the other
+  if (std::max(h->EZ, h->EG) <= 16) return false;
+  if (D && C) return h->Gn <= 256 || M.N >= kBigTokensWideIn;
+  return h->Gn + h->Gm >= kBigGroups && (ops == FRAMEFB_OP_FORWARD || M.N >= kBigTokensOne);
 }
 
 struct GrpLaunches {
@@ -367,18 +387,25 @@ framefb_status grp_check(const framefb_mat* mats, int32_t nmats, int32_t ops, fr
                          GrpReady* keep) {
   *ws_need = 0;
   if (nmats == 0) return FRAMEFB_OK;
-  for (int32_t j = 0; j < nmats; ++j) {
-    framefb_status s = check_mat(mats[j], ops, dt);
-    if (s != FRAMEFB_OK) return s;
-    // the workspace asked for covers fewer tokens too, where the contraction
-    // path takes these plans (kMinTokensWideIn)
-    if (dt == FRAMEFB_BF16 && header_of(mats[j].plan)->Gn > 128 && mats[j].ldx == mats[j].n && mats[j].ldy == mats[j].m) {
-      size_t need = 0;
-      s = dense_check(&mats[j], 1, ops, dt, &need);
+  int64_t pairs = 0, slots = 0;
+  int32_t stride = 0;
+  bool big = false;
+  std::vector<framefb_mat> wide;  // unpadded, with an input side that fewer tokens send to the contraction path
+  try {
+    for (int32_t j = 0; j < nmats; ++j) {
+      const framefb_status s = check_mat(mats[j], ops, dt);
       if (s != FRAMEFB_OK) return s;
-      *ws_need = std::max(*ws_need, need);
+      const FfbPlanHeader* h = header_of(mats[j].plan);
+      pairs += (mats[j].N + 1) / 2;
+      stride = std::max(stride, (h->nnz + 63) & ~63);
+      if (dt == FRAMEFB_BF16 && h->Gn > 128 && mats[j].ldx == mats[j].n && mats[j].ldy == mats[j].m) wide.push_back(mats[j]);
     }
+  } catch (const std::bad_alloc&) {
+    return FRAMEFB_ENOMEM;
   }
+  // (asked for at every token count, as on the contraction path)
+  const framefb_status ds = dense_check(wide.data(), static_cast<int32_t>(wide.size()), ops, dt, ws_need);
+  if (ds != FRAMEFB_OK) return ds;
   try {
     auto all = std::make_shared<GrpLaunches>();
     for (const Chunk& c : chunks_of(mats, nmats)) {
@@ -387,11 +414,18 @@ framefb_status grp_check(const framefb_mat* mats, int32_t nmats, int32_t ops, fr
       l.P = l.b.prep();
       const framefb_status s = prepare(c, ops, dt, l.P);
       if (s != FRAMEFB_OK) return s;
-      *ws_need = std::max(*ws_need, keep ? l.P.ws_bytes : l.P.ws_cover);
+      *ws_need = std::max(*ws_need, l.P.ws_bytes);
+      slots = std::max(slots, l.P.slots);
+      big = big || l.P.v.big;
       l.fn = kernel_ptr(l.P.v, dt);
       l.mats = static_cast<unsigned>(c.mats.size());
       l.reduce = (ops & FRAMEFB_OP_GRAD_COEFF) && l.P.nnz_max > 0;
     }
+    // What a query reports covers any smaller token count too: more tokens can make
+    // fewer, larger units, and calls of few tokens take other kernels, with a CTA per
+    // SM, where the plan is a big one.
+    if (!keep && (ops & FRAMEFB_OP_GRAD_COEFF))
+      *ws_need = std::max(*ws_need, static_cast<size_t>((big ? slots : std::min(slots, pairs)) + nmats) * stride * sizeof(float) + 256);
     if (keep) *keep = std::move(all);
   } catch (const std::bad_alloc&) {
     return FRAMEFB_ENOMEM;

@@ -9,8 +9,11 @@
 
 namespace ffb_host {
 
-// Whether a matrix of a call runs on the group-transform kernel.
-bool grp_takes(const framefb_mat& M, int32_t ops, framefb_dtype dt);
+// Whether a plan fits the group-transform kernel, with whole or compacted buffers,
+// and whether a matrix of a call, of a plan of this kind, runs on it.
+enum class GrpKind { none, whole, big };
+GrpKind grp_kind(const framefb_plan* plan);
+bool grp_takes(GrpKind kind, const framefb_mat& M, int32_t ops, framefb_dtype dt);
 
 // The launches of a call, with their parameters filled.
 struct GrpLaunches;

@@ -113,3 +113,41 @@ def test_fp32_one_phase_kernel(mats, N, nnz, kernel, monkeypatch):
     monkeypatch.setenv("FRAMEFB_KERNEL", "")
     if nnz <= 8192:
         assert names(b, ALL) == ["fft_tile_kernel<7>"]
+
+
+# fp32 plans in compacted buffers: wide sides with short columns stay on the
+# one-phase kernel; long columns leave it where both gradients are asked for, or
+# (8192 features and more in all) for a forward pass, or for many tokens
+@pytest.mark.parametrize("shape,N,nnz,fused,forward,dx", [((8448, 64), 5, 300, "phase", "phase", "phase"),
+                                                          ((256, 256), 9, 6000, "tile", "phase", "phase"),
+                                                          ((4096, 4096), 5, 4608, "tile", "tile", "phase"),
+                                                          ((4096, 4096), 800, 4608, "tile", "tile", "tile")])
+def test_fp32_compacted_buffers(shape, N, nnz, fused, forward, dx):
+    b = AdapterBatch(load([shape], N, nnz, "f32"), DEV, ops=ALL)
+    for ops, kernel in ((ALL, fused), (F, forward), (ffb.OP_BACKWARD_DX, dx)):
+        assert names(b, ops) == [f"fft_{kernel}_kernel<{ops}>"]
+    if max(shape) > 256:
+        return
+    e, x = Expect(b, 0), b.bufs[0]
+    X, dY = host64(x.X), host64(x.dY)
+    b.run(F)
+    b.run(ffb.OP_BACKWARD_DX)
+    torch.cuda.synchronize()
+    assert_f32(host64(x.Y), e.y(X, np.zeros((N, shape[1]))), what="Y")
+    assert_f32(host64(x.dX), e.dx(dY, np.zeros((N, shape[0]))), what="dX")
+
+
+def test_one_workspace_serves_fewer_tokens_of_wide_plans():
+    """Wide bf16 plans run as contractions below 128 tokens (unpadded rows) or on the
+    warp-MMA kernel (padded rows), fp32 ones with long columns on the one-phase kernel
+    below 768: the workspace of more tokens serves them."""
+    for dtype, shape, pad, Ns in (("bf16", (4608, 64), 0, (1, 64, 127, 128, 300)), ("bf16", (4608, 64), 16, (1, 64, 127, 128, 300)),
+                                  ("f32", (4096, 4096), 0, (1, 100, 767, 768))):
+        kw = {"support_mode": wl.ZIPF_ROWS} if dtype == "bf16" else {}
+        b = AdapterBatch(load([shape], max(Ns), 4300 if dtype == "bf16" else 4608, dtype, **kw), DEV, ops=ALL)
+        sizes = []
+        for N in Ns:
+            c = ffb.framefb_mat.from_buffer_copy(b.mats[0])
+            c.N, c.ldx, c.ldy = N, c.ldx + pad, c.ldy + pad
+            sizes.append(ffb.framefb_workspace_size([c], ALL if dtype == "bf16" else ffb.OP_GRAD_COEFF))
+        assert sizes == sorted(sizes), (dtype, shape, pad, sizes)
