@@ -36,7 +36,7 @@ namespace grp {
 using namespace pair;
 
 // Bounded by construction: this kernel waits on nothing but CTA barriers.
-constexpr int kMaxMats = 96;  // matrices of a launch
+constexpr int kMaxMats = 160;  // matrices of a launch
 
 // Buffers of a token pair (float2 offsets), side 0 the input side (X, V, RG,
 // dX), side 1 the output side (dY, U, RZ, Y): A[s] V or U, B[s] RG or RZ.

@@ -337,7 +337,7 @@ __device__ __forceinline__ void flush_dc(const uint8_t* plan, float* dst, const 
 
 // dC_q = seff * sum over the CTAs that visited the matrix, in a fixed order:
 // kLanes interleaved sums, then a tree over them.
-constexpr int kReduceMats = 96;
+constexpr int kReduceMats = 160;
 struct ReduceMat {
   float* dC;
   int32_t c0, c1, nnz;  // CTAs [c0, c1] visited the matrix

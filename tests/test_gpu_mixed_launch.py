@@ -1,5 +1,5 @@
 """One launch of the group kernel over matrices of unlike cost, over plans of their
-own, and fewer units than CTAs: results against the fp64 oracle (fp32 bar), and a
+own, with fewer units than CTAs, and more matrices than one launch holds: results against the fp64 oracle (fp32 bar), and a
 workspace that serves every smaller token count."""
 import numpy as np
 import pytest
@@ -55,7 +55,8 @@ def test_one_workspace_serves_fewer_tokens(mats, nnz):
 
 @pytest.mark.parametrize("mats,nnz,N,kw", [(MIXED, 1000, 203, {}), (UNLIKE, 500, 1, {}), (UNLIKE, 500, 64, {}),
                                            (UNLIKE, 500, 333, {}), ([(256, 256)] * 20, 128, 9, {"per_layer_support": True}),
-                                           ([(512, 256)] * 9, 3000, 5, {"per_layer_support": True})])
+                                           ([(512, 256)] * 9, 3000, 5, {"per_layer_support": True}),
+                                           ([(64, 96)] * 163, 40, 3, {})])
 def test_parity(mats, nnz, N, kw):
     b = load(mats, N, nnz, **kw)
     b.run(ALL, b.workspace(ALL))
