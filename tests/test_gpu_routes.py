@@ -151,3 +151,19 @@ def test_one_workspace_serves_fewer_tokens_of_wide_plans():
             c.N, c.ldx, c.ldy = N, c.ldx + pad, c.ldy + pad
             sizes.append(ffb.framefb_workspace_size([c], ALL if dtype == "bf16" else ffb.OP_GRAD_COEFF))
         assert sizes == sorted(sizes), (dtype, shape, pad, sizes)
+
+
+def test_contractions_over_more_than_a_chunk_of_tokens():
+    """T-block frames have no transform kernel: more tokens than the contraction path
+    holds at a time (8192), dC summed over both chunks."""
+    w = wl.WORKLOADS["tblock_tff"]
+    N = 8192 + 77
+    b = AdapterBatch(w, DEV, N=N, indices=[0, 1], ops=ALL)
+    assert "dense_gemm_kernel<bf16_hilo>" in names(b, ALL) and not any(k.startswith("row") for k in names(b, ALL))
+    b.run(ALL, b.workspace(ALL))
+    torch.cuda.synchronize()
+    for j, x in enumerate(b.bufs):
+        e, X, dY = Expect(b, j), host64(x.X), host64(x.dY)
+        assert_bf16(host64(x.Y), e.y(X, np.zeros((N, x.spec.m))), what=f"Y[{j}]")
+        assert_bf16(host64(x.dX), e.dx(dY, np.zeros((N, x.spec.n))), what=f"dX[{j}]")
+        assert_bf16(host64(x.dC), e.dc(X, dY), what=f"dC[{j}]")
