@@ -898,8 +898,8 @@ extern "C" framefb_status framefb_run(const framefb_mat* mats, int32_t nmats, in
   std::vector<framefb_mat> den, row, fft;
   framefb_status s = plan_waves(mats, nmats, ops, dtype, waves, den, row, fft);
   if (s != FRAMEFB_OK) return s;
-  // validate everything before queueing anything; the waves and the two
-  // paths run one after the other on the stream and share the workspace
+  // validate everything before queueing anything; the waves and the other
+  // paths run one after another on the stream and share the workspace
   size_t need = 0;
   std::vector<Ready> ready;
   for (const std::vector<framefb_mat>& w : waves) {

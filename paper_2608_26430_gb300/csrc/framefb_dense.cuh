@@ -1,6 +1,7 @@
 // Device code of the dense path of libframefb: frames outside the structured
-// kernels (the paper's rho = 2 regime, where Phi is a dense realified DFT of
-// size d/2, and redundant frames with T blocks, k*rho > d).  Phi is treated
+// kernels and the row transform (redundant frames with T blocks, k*rho > d, and
+// rho = 2 frames whose DFT size, token count or plan framefb_row.cu leaves here),
+// and structured bf16 plans that no other path takes.  Phi is treated
 // as a dense d x K matrix (K = k*rho frame columns), so one pass of the
 // adapter is three contractions around the coefficient SpMM (Sec. 3.1
 // update, Lemma 1 gradient of Appendix A):

@@ -113,16 +113,13 @@ Variant variant(const FfbPlanHeader* h) {
 }
 
 void* kernel_ptr(const Variant& v, framefb_dtype dt) {
-#define FFB_GRP(N, E, B)                                                                             \
-  if (v == Variant{N, E, B})                                                                         \
-    return dt == FRAMEFB_BF16 ? reinterpret_cast<void*>(fg::fft_tile_kernel<__nv_bfloat16, N, E, B>)    \
-                              : reinterpret_cast<void*>(fg::fft_tile_kernel<float, N, E, B>);
-  FFB_GRP(256, 4, false)
-  FFB_GRP(256, 8, false)
-  FFB_GRP(512, 8, false)
-  FFB_GRP(512, fg::kBigE, true)
-#undef FFB_GRP
-  return nullptr;
+  const Variant big{512, fg::kBigE, true};
+  if (dt == FRAMEFB_BF16)  // (plans with whole buffers run on the tcgen05 kernels)
+    return v == big ? reinterpret_cast<void*>(fg::fft_tile_kernel<__nv_bfloat16, 512, fg::kBigE, true>) : nullptr;
+  if (v == Variant{256, 4, false}) return reinterpret_cast<void*>(fg::fft_tile_kernel<float, 256, 4, false>);
+  if (v == Variant{256, 8, false}) return reinterpret_cast<void*>(fg::fft_tile_kernel<float, 256, 8, false>);
+  if (v == Variant{512, 8, false}) return reinterpret_cast<void*>(fg::fft_tile_kernel<float, 512, 8, false>);
+  return v == big ? reinterpret_cast<void*>(fg::fft_tile_kernel<float, 512, fg::kBigE, true>) : nullptr;
 }
 
 struct Prepared {

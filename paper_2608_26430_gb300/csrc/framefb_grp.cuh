@@ -16,17 +16,17 @@
 //             RZ / RG, dC in registers.
 // The rows of the next unit are prefetched to L2 in phase B.
 //
-// BIG: plans of more than 16 entries per column (8192-entry supports).  The
-// buffers hold only the coefficients that the support names (the popcount of
-// the group's mask below a coefficient is its slot), so that pairs of 14336-wide
-// rows fit, and the coefficient values and dC sums sit in shared memory.
+// BIG: plans of more than 16 entries per column (8192-entry supports) or of more
+// coefficients than whole buffers hold.  The buffers hold only the coefficients
+// that the support names (the popcount of the group's mask below a coefficient is
+// its slot), so that pairs of 14336-wide rows fit where the support leaves most
+// of them out (Zipf rows; 8192 uniform entries name too many), and the coefficient
+// values and dC sums sit in shared memory.
 //
-// Bound: latency.  768 <-> 3072 in bf16: 3.1 k shared-memory and L1 wavefronts
-// and 7 k instructions per token pair against 5.9 k cycles (issue 35 %, a third
-// of the stalls at the barriers between the phases); a 4096 -> 14336 BIG pair
-// 19 k wavefronts in 40 k cycles.  Measured (fused pass, against the kernels
-// that ran before): fp32, 8 matrices of 768^2, 2048 tokens 202 -> 107 us; a
-// LLaMA-3-8B-shaped layer, 16384 tokens 5.92 -> 4.07 ms.
+// Bound: latency: two phases with a barrier between them, one or two CTAs per SM.
+// Measured (fused pass, against the kernels that ran before): fp32, 8
+// matrices of 768^2, 2048 tokens 203 -> 104 us; a LLaMA-3-8B-shaped layer, Zipf
+// supports, 16384 tokens 5.90 -> 4.07 ms.
 #pragma once
 #include "framefb_pair.cuh"
 
