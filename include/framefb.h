@@ -132,6 +132,9 @@ void framefb_frame_free(framefb_frame* f);
  * T blocks (k*rho > d) -- runs on the dense path, which treats Phi as a
  * dense d x ncols matrix and reads it from `dense`: a device copy, byte for
  * byte, of the image framefb_frame_dense_pack() writes (16-byte aligned).
+ * (Frames with rho = 2 of common sizes run as FFTs on chip instead, from a
+ * token count on that depends on the size; calls ask for the same image and
+ * workspace either way.)
  * `dense` may be NULL for structured frames.
  */
 typedef struct {
@@ -218,7 +221,8 @@ void framefb_plan_free(framefb_plan* plan);
  * row, and rounding the bf16 output once per part would exceed the bf16
  * tolerance on heavy-tailed supports: such plans have no parts.)  Every part is a plan of its own over its two blocks,
  * stored in the plan's device image after the whole plan, with the list of
- * its entries' indices into the caller's C values and dC (int32).  framefb_run
+ * its entries' indices into the caller's C values and dC (int32).  Where no
+ * other kernel takes the whole plan (or is slower), framefb_run
  * runs each part as a matrix of the fused kernels: ΔW is linear in C, so
  * Y and dX take the sum of the parts' contributions, and each part writes
  * its own entries of dC.  This restates the method exactly; it is the
