@@ -66,3 +66,22 @@ def test_parity(mats, nnz, N, kw):
         assert_f32(host64(x.Y), e.y(X, np.zeros((N, x.spec.m))), what=f"Y[{j}]")
         assert_f32(host64(x.dX), e.dx(dY, np.zeros((N, x.spec.n))), what=f"dX[{j}]")
         assert_f32(host64(x.dC), e.dc(X, dY), what=f"dC[{j}]")
+
+
+def test_dc_sums_are_as_accurate_as_the_one_phase_kernels(monkeypatch):
+    """dC over many tokens per CTA: no further from fp64 than the one-phase kernel's on
+    the same inputs, over the entries of all matrices (both kernels sum in fp32; what
+    differs is the number of roundings along a sum)."""
+    err = {}
+    for kernel in ("", "tile"):
+        monkeypatch.setenv("FRAMEFB_KERNEL", kernel)
+        b = load([(768, 768)] * 8, 2048, 1000)
+        b.run(ffb.OP_GRAD_COEFF, b.workspace(ffb.OP_GRAD_COEFF))
+        torch.cuda.synchronize()
+        num = den = 0.0
+        for j, x in enumerate(b.bufs):
+            ref = Expect(b, j).dc(host64(x.X), host64(x.dY))
+            num += np.sum((host64(x.dC) - ref) ** 2)
+            den += np.sum(ref ** 2)
+        err[kernel] = np.sqrt(num / den)
+    assert err[""] <= err["tile"], err
