@@ -17,10 +17,10 @@
 //               of Y / dX (prefetched to L2 before the SpMM).
 // (Token pairs: framefb_pair.cuh.)
 //
-// Bound: shared memory.  At d = 4096 a token pair moves about 13 k wavefronts
-// (four transforms of four passes and the SpMM's gathers), against 9 k issue
-// cycles and 32 KB of DRAM traffic; the pair takes 23 k cycles, one CTA of 512
-// threads per SM.  Measured (fused pass): 4 matrices of 4096^2, 8192 tokens
+// Bound: shared memory.  At d = 4096 a token pair moves about 15 k wavefronts
+// (four transforms of four passes and the SpMM's gathers; 3 k of them bank
+// conflicts), against 10 k issue cycles and 80 KB of DRAM traffic; the pair takes
+// 23 k cycles, one CTA of 512 threads per SM.  Measured (fused pass): 4 matrices of 4096^2, 8192 tokens
 // 1.21 ms against 6.90 ms as dense contractions; 24 of 768^2, 4096 tokens
 // 0.57 ms against 2.99 ms.  dC against the fp64 oracle: 3e-7 relative (1.7e-5
 // before: bf16 hi + lo frames).
