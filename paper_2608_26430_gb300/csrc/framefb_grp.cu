@@ -131,6 +131,11 @@ struct Prepared {
   size_t smem, ws_bytes;
 };
 
+// Matrices of a launch of big plans: the dC sums of 8192 entries each (a slot per CTA
+// and matrix) then fit the library's static workspace.
+constexpr int kMaxBig = 96;
+static_assert((152 + kMaxBig) * 8192 * 4 + 256 <= FRAMEFB_STATIC_WS_BYTES, "static workspace");
+
 // One launch: as many matrices as the parameters hold, of one variant.
 struct Chunk {
   std::vector<const framefb_mat*> mats;
@@ -156,7 +161,7 @@ std::vector<Chunk> chunks_of(const framefb_mat* mats, int32_t nmats) {
       if (mats[j].plan != plan) shape_of(header_of(plan = mats[j].plan), v, sh);
       Regions with = all;
       with.take(sh, 1, v);
-      if (!open || static_cast<int>(out.back().mats.size()) == fg::kMaxMats || with.bytes(v) > budget(v)) {
+      if (!open || static_cast<int>(out.back().mats.size()) == (v.big ? kMaxBig : fg::kMaxMats) || with.bytes(v) > budget(v)) {
         out.push_back(Chunk{{}, v});
         with = Regions();
         with.take(sh, 1, v);

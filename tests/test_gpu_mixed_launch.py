@@ -85,3 +85,15 @@ def test_dc_sums_are_as_accurate_as_the_one_phase_kernels(monkeypatch):
             den += np.sum(ref ** 2)
         err[kernel] = np.sqrt(num / den)
     assert err[""] <= err["tile"], err
+
+
+def test_many_big_plans_fit_the_static_workspace():
+    w = wl.Workload("big", tuple(wl.MatSpec(f"w{i}", 256, 4608) for i in range(110)), N=40, nnz=8192, dtype="bf16",
+                    c_std=0.02, support_mode=wl.ZIPF_ROWS)
+    b, ref = (AdapterBatch(w, DEV, ops=ALL, alias_inputs=True) for _ in range(2))
+    assert ffb.framefb_kernel_names(b.mats, ALL, b.dtype_code) == ["fft_tile_kernel<7>"]
+    ffb.framefb_run_static_ws(b.mats, ALL, b.dtype_code)
+    ref.run(ALL, ref.workspace(ALL))
+    torch.cuda.synchronize()
+    for x, y in zip(b.bufs, ref.bufs):
+        assert torch.equal(x.Y, y.Y) and torch.equal(x.dX, y.dX) and torch.equal(x.dC, y.dC)
